@@ -464,12 +464,13 @@ static size_t workspace_rule(int dir, const ct_geometry *g, ct_projector proj, c
         case CT_SF:
             if (nc) return ctp::nc_footprint_fits(G, 0) ? vox * isz : 0;
             return G.max_m_sf_u <= 3.5f && zmajor ? vox * isz : 0;
-        default:  // SF-TT: streaming forward in circular flat 3D geometry, footprint forward otherwise
+        default:  // SF-TT: none in fan beam; streaming forward in circular flat 3D geometry, footprint forward otherwise
+            if (G.is2d) return 0;
             return ctp::sftt_circ_fits(G) ? (zmajor ? vox * isz : 0) : vox * isz;
         }
     }
     switch (proj) {
-    case CT_RAY: return nc ? 0 : cells * 4;
+    case CT_RAY: return nc || G.is2d ? 0 : cells * 4;
     case CT_DD: return !nc || ctp::nc_footprint_fits(G, 1) ? cells * 4 : 0;
     case CT_SF_TT: return cells * 4;
     default: return 0;

@@ -30,6 +30,14 @@ cudaError_t launch_sftt_circ(int dir, const CtGrid &g, const CtView *views, int 
                              void *out, int batch, cudaStream_t st);
 cudaError_t launch_nc(int kind, int dir, const CtGrid &g, const CtView *views, int in_t, const void *in,
                       int out_t, void *out, int batch, cudaStream_t st);
+// 2D fan beam (k_fan.cu): every projector, dir 0 forward, 1 back (DD and SF-TT
+// take the sinogram already scaled by each cell's factor), 2 the recon-mode
+// back of SF, DD and voxel-driven.  fan_fits: 2D, and forward footprints of at
+// most 8 cells (wider ones take the general forward of k_sf.cu).
+enum FanKind { FAN_SF = 0, FAN_DD = 1, FAN_TT = 2, FAN_VOX = 3, FAN_RAY = 4 };
+bool fan_fits(const CtGrid &g, int kind, int dir);
+cudaError_t launch_fan(int kind, int dir, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
+                       void *out, int batch, cudaStream_t st);
 // voxel-driven forward in circular geometry (the streaming forward of k_sf.cu)
 cudaError_t launch_vx_fwd_circ(const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                                void *out, int batch, cudaStream_t st);

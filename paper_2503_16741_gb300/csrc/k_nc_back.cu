@@ -185,6 +185,7 @@ tt_prescale(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
 cudaError_t launch_sftt(int dir, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                         void *out, int batch, cudaStream_t st) {
     const bool circ = sftt_circ_fits(g);
+    if (dir == 0 && fan_fits(g, FAN_TT, 0)) return launch_fan(FAN_TT, 0, g, views, in_t, in, out_t, out, batch, st);
     if (dir == 0)
         return circ ? launch_sftt_circ(0, g, views, in_t, in, out_t, out, batch, st)
                     : launch_nc(NC_TT, 0, g, views, in_t, in, out_t, out, batch, st);
@@ -204,8 +205,9 @@ cudaError_t launch_sftt(int dir, const CtGrid &g, const CtView *views, int in_t,
     }
     e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = circ ? launch_sftt_circ(1, g, views, 0, yp, out_t, out, batch, st)
-                 : launch_nc(NC_TT, 1, g, views, 0, yp, out_t, out, batch, st);
+        e = g.is2d ? launch_fan(FAN_TT, 1, g, views, 0, yp, out_t, out, batch, st)
+            : circ ? launch_sftt_circ(1, g, views, 0, yp, out_t, out, batch, st)
+                   : launch_nc(NC_TT, 1, g, views, 0, yp, out_t, out, batch, st);
     const cudaError_t ef = workspace_free(yp, st);
     return e != cudaSuccess ? e : ef;
 }

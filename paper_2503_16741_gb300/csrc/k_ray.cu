@@ -493,6 +493,7 @@ cudaError_t ray_launch_t(int dir, const CtGrid &g, const CtView *views, const vo
 
 cudaError_t launch_ray(int dir, const CtGrid &g, const CtView *views, int in_t, const void *in,
                        int out_t, void *out, int batch, cudaStream_t st) {
+    if (g.is2d) return launch_fan(FAN_RAY, dir, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return ray_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return ray_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);

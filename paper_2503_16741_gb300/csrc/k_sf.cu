@@ -1184,6 +1184,14 @@ cudaError_t sf_launch_t(int dir, const CtGrid &g, const CtView *views, const voi
                   : fp_back_circ<TIn, false, false>(g, views, src, out, out_t, batch, st);
 }
 
+// DD back from the scaled sinogram, fan beam and circular geometry
+cudaError_t dd_back_scaled(const CtGrid &g, const CtView *views, const float *yp, void *out, int out_t, int batch,
+                           cudaStream_t st) {
+    if (g.is2d) return launch_fan(FAN_DD, 1, g, views, 0, yp, out_t, out, batch, st);
+    return g.variant == GEO_CIRC_CURVED ? fp_back_circ<float, true, true>(g, views, yp, out, out_t, batch, st)
+                                        : fp_back_circ<float, false, true>(g, views, yp, out, out_t, batch, st);
+}
+
 // DD in circular geometry; the back direction scales the sinogram by L_c
 // into a stream-ordered FP32 workspace first
 template <typename TIn>
@@ -1204,9 +1212,7 @@ cudaError_t dd_launch_t(int dir, const CtGrid &g, const CtView *views, const voi
     else
         dd_prescale<TIn, false><<<blocks, 256, 0, st>>>(g, views, src, yp, batch);
     e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = curved ? fp_back_circ<float, true, true>(g, views, yp, out, out_t, batch, st)
-                   : fp_back_circ<float, false, true>(g, views, yp, out, out_t, batch, st);
+    if (e == cudaSuccess) e = dd_back_scaled(g, views, yp, out, out_t, batch, st);
     const cudaError_t ef = workspace_free(yp, st);
     return e != cudaSuccess ? e : ef;
 }
@@ -1269,8 +1275,7 @@ cudaError_t launch_dd_back_scratch(const CtGrid &g, const CtView *views, int in_
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return curved ? fp_back_circ<float, true, true>(g, views, scratch, out, out_t, batch, st)
-                  : fp_back_circ<float, false, true>(g, views, scratch, out, out_t, batch, st);
+    return dd_back_scaled(g, views, scratch, out, out_t, batch, st);
 }
 
 namespace {
@@ -1304,6 +1309,7 @@ cudaError_t recon_fp_t(int dd, const CtGrid &g, const CtView *views, const void 
 cudaError_t launch_recon_fp(int dd, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                             void *out, int batch, cudaStream_t st) {
     if (g.variant == GEO_NONCIRC_FLAT) return launch_nc_recon(dd, g, views, in_t, in, out_t, out, batch, st);
+    if (g.is2d) return launch_fan(dd ? FAN_DD : FAN_SF, 2, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return recon_fp_t<float>(dd, g, views, in, out, out_t, batch, st);
     case 1: return recon_fp_t<__half>(dd, g, views, in, out, out_t, batch, st);
@@ -1363,6 +1369,7 @@ cudaError_t launch_sf(int dir, const CtGrid &g, const CtView *views, int in_t, c
                       int out_t, void *out, int batch, cudaStream_t st) {
     if (g.variant == GEO_NONCIRC_FLAT && nc_footprint_fits(g, 0))
         return launch_nc(0, dir, g, views, in_t, in, out_t, out, batch, st);
+    if (fan_fits(g, FAN_SF, dir)) return launch_fan(FAN_SF, dir, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return sf_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return sf_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);
@@ -1381,6 +1388,7 @@ cudaError_t launch_dd(int dir, const CtGrid &g, const CtView *views, int in_t, c
         default: return dd_nc_back<__nv_bfloat16>(g, views, in, out, out_t, batch, st);
         }
     }
+    if (dir == 0 && fan_fits(g, FAN_DD, 0)) return launch_fan(FAN_DD, 0, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return dd_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return dd_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);

@@ -1,0 +1,71 @@
+"""The fan-beam kernels at the edges of their tiles (8 x 4 pixel patches, 32
+cells, 8 view groups of 64 staged views, runs of slabs), against the FP64
+oracle at the FP32 path's bound, in every projector and direction."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+import workloads as W
+from gpu_util import TOL_F32, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ct():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_16741_gb300 as ct
+    ct.load()
+    return ct
+
+
+# nx, ny, nu, views, cell size (mm): one pixel; single rows and columns; one past and one short of a tile; more
+# views than one staging; wide footprints (5 to 8 cells, and beyond 8); a detector narrower than a footprint
+SIZES = [(1, 1, 5, 1, 3.0), (33, 1, 31, 7, 2.0), (1, 29, 40, 9, 2.0), (8, 4, 32, 8, 1.5), (9, 5, 33, 65, 1.7),
+         (40, 67, 129, 131, 1.9), (31, 31, 150, 12, 0.85), (12, 12, 160, 10, 0.4), (17, 16, 2, 6, 4.0)]
+
+
+def _spec(det, nx, ny, nu, views, du):
+    return W.GeometrySpec("fan2d", det, nx, ny, 1, 1.6, 1.6, 1.0, nu, 1, du, 1.0, views,
+                          theta=0.2 + 2 * np.pi * np.arange(views) / views, sad=300.0, sdd=610.0, x_src=1.5,
+                          u_ofst=0.7, x_ofst=-1.0, y_ofst=2.0)
+
+
+def _same(got, ref, what):
+    if np.linalg.norm(ref) == 0:
+        assert float(np.abs(got).max()) == 0, what
+    else:
+        assert rel_l2(got, ref) <= TOL_F32, what
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("size", SIZES, ids=["x".join(map(str, s)) for s in SIZES])
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel", "ray", "sftt"])
+def test_fan_pair_matches_oracle(ct, det, size, proj):
+    spec = _spec(det, *size)
+    g = ct.Geometry.from_spec(spec)
+    x, y = W.random_volume(spec, seed=1, batch=2), W.random_sino(spec, seed=2, batch=2)
+    xd = torch.as_tensor(x[:, 0], dtype=torch.float32).cuda()
+    yd = torch.as_tensor(y[:, :, 0], dtype=torch.float32).cuda()
+    if proj == "sftt" and (det == "curved" or size[4] < 0.5):
+        with pytest.raises(ct.CTError):
+            ct.forward(g, xd, proj)
+        return
+    Ax, Aty = ct.forward(g, xd, proj), ct.back(g, yd, proj)
+    for b in range(2):
+        _same(Ax[b].cpu().numpy(), oracle.forward(spec, proj, x[b]).reshape(g.sino_shape), "forward")
+        _same(Aty[b].cpu().numpy(), oracle.back(spec, proj, y[b]).reshape(g.vol_shape), "back")
+    assert torch.equal(Ax[1], ct.forward(g, xd[1], proj)) and torch.equal(Aty[1], ct.back(g, yd[1], proj))
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("proj", ["voxel", "dd", "sf"])
+def test_fan_recon_back_matches_oracle(ct, det, proj):
+    spec = _spec(det, 40, 67, 129, 131, 1.9)
+    g = ct.Geometry.from_spec(spec)
+    q = W.random_sino(spec, seed=3)[0]
+    got = ct.back(g, torch.as_tensor(q[:, 0], dtype=torch.float32).cuda(), proj, mode="recon")
+    _same(got.cpu().numpy(), oracle.back_recon(spec, q, proj).reshape(g.vol_shape), proj)
