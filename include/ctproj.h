@@ -22,15 +22,16 @@
  * stream-ordered workspace from a library-owned memory pool on the current
  * device (kept in the pool between calls, so steady-state calls do not reach
  * the driver's allocator) and return it on the same stream:
- *   ct_back with CT_DD or CT_SF_TT, and with CT_RAY in circular geometry:
+ *   ct_back with CT_DD or CT_SF_TT, and with CT_RAY in circular cone-beam
+ *     geometry:
  *     the sinogram scaled by each cell's path length, amplitude or secant,
  *     batch x nview x nv x nu floats (non-circular CT_DD only when its
  *     footprints fit the footprint kernels, at most 8 cells by 4 rows);
- *   ct_forward with CT_SF or CT_DD (circular geometry with nz a multiple
- *     of 4 and at least 8, or non-circular geometry), with CT_SF_TT, and
- *     with CT_VOXEL (the same circular cases): a z-major copy of the volume,
- *     batch x nz x ny x nx elements of in_t (skipped, at some speed, when it
- *     cannot be had).
+ *   ct_forward with CT_SF, CT_DD or CT_SF_TT (cone beam) and with CT_VOXEL
+ *     (circular cone beam): a reordered copy of the volume, batch x nz x ny x
+ *     nx elements of in_t; in circular geometry with nz rounded up to a
+ *     multiple of 4, twice that for CT_SF, CT_DD and CT_VOXEL, and none below 4
+ *     slices (skipped, at some speed, when it cannot be had).
  * ct_workspace_bytes gives that size for a call; ct_workspace_limit caps
  * what the pool keeps once calls have returned it.
  * Results are deterministic: no atomics, fixed summation order.

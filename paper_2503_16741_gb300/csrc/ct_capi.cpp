@@ -452,21 +452,22 @@ static size_t workspace_rule(int dir, const ct_geometry *g, ct_projector proj, c
     const size_t cells = (size_t)g->nview * g->nv * g->nu * (size_t)batch;
     const size_t isz = in_t == CT_F32 ? 4 : 2;
     const bool nc = G.variant == ctp::GEO_NONCIRC_FLAT;
-    const bool zmajor = !G.is2d && g->nz % 4 == 0 && g->nz >= 8;  // the streaming forward's copy
+    // the circular SF-TT forward's z-major copy (columns padded to four voxels)
+    const size_t zvox = (size_t)g->nx * g->ny * ctp::zmajor_pitch(G) * (size_t)batch;
     if (mode == CT_MODE_RECON) return 0;
     if (dir == 0) {
         switch (proj) {
-        case CT_VOXEL: return !nc && zmajor ? vox * isz : 0;
+        case CT_VOXEL: return ctp::circ_fwd_fits(G, ctp::BK_VOX, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;
         case CT_RAY: return 0;
         case CT_DD:
             if (nc) return ctp::nc_footprint_fits(G, 1) ? vox * isz : 0;
-            return G.max_m_dd_u <= 3.5f && zmajor ? vox * isz : 0;
+            return ctp::circ_fwd_fits(G, ctp::BK_DD, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;
         case CT_SF:
             if (nc) return ctp::nc_footprint_fits(G, 0) ? vox * isz : 0;
-            return G.max_m_sf_u <= 3.5f && zmajor ? vox * isz : 0;
+            return ctp::circ_fwd_fits(G, ctp::BK_SF, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;
         default:  // SF-TT: none in fan beam; streaming forward in circular flat 3D geometry, footprint forward otherwise
             if (G.is2d) return 0;
-            return ctp::sftt_circ_fits(G) ? (zmajor ? vox * isz : 0) : vox * isz;
+            return ctp::sftt_circ_fits(G) ? (ctp::zmajor_copy_fits(G, batch) ? zvox * isz : 0) : vox * isz;
         }
     }
     switch (proj) {

@@ -208,6 +208,76 @@ __device__ __forceinline__ void split_cell(float f, int &ref, float &frac) {
     frac = f - r;
 }
 
+// 1 / x for finite x != 0 far from the ends of the exponent range: the
+// hardware's approximation improved by one Newton-Raphson step r (2 - x r)
+// (three instructions; within an ulp of the correctly rounded value)
+__device__ __forceinline__ float rcp_newton(float x) {
+    const float r = __fdividef(1.f, x);
+    return fmaf(r, fmaf(-x, r, 1.f), r);
+}
+
+// Angle of the direction (den, num), den > 0: the first terms of arctan's
+// Taylor series for the slopes below 1/16 that a voxel's corners have as seen
+// from the source (next term 2.6e-11 relative), the library function beyond.
+__device__ __forceinline__ float slope_angle(float num, float den) {
+    const float q = __fdividef(num, den), q2 = q * q;
+    if (q2 > 1.f / 256.f) return atan2f(num, den);
+    return q * fmaf(q2, fmaf(q2, fmaf(q2, -1.f / 7.f, 0.2f), -1.f / 3.f), 1.f);
+}
+
+// Transaxial footprint of a column whose centre lies at (cu, cn) in the
+// detector frame: nearest cell aref and the four knots relative to it.  The
+// corners come in pairs opposite about the centre, so each pair shares its
+// numerator, one of its knots lies below the centre and the other above, and
+// the four sort with min and max alone.  (Four fast divisions of about one
+// cell: ~1e-7 cell each.)
+template <bool CURVED, bool DD>
+__device__ __forceinline__ void column_knots(const CtView &V, float cu, float cn, int &aref, float (&k)[4]) {
+    float fr, lo[2], hi[2];
+    constexpr int NP = DD ? 1 : 2;
+    float pu[2], pn[2];  // one corner of each pair (DD: a boundary point on the non-main axis)
+    if (DD) {
+        const int q = V.main_y ? 0 : 1;
+        pu[0] = 0.5f * V.au[q];
+        pn[0] = 0.5f * V.an[q];
+    } else {
+        pu[0] = V.cdu[3]; pn[0] = V.cdn[3];
+        pu[1] = V.cdu[1]; pn[1] = V.cdn[1];
+    }
+    if (CURVED) {
+        split_cell(fmaf(V.Ku, atan2f(cu, cn), V.Cu), aref, fr);
+        const float rho2 = fmaf(cu, cu, cn * cn);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const float num = fmaf(pu[p], cn, -cu * pn[p]), dot = fmaf(pu[p], cu, pn[p] * cn);
+            const float t1 = fmaf(V.Ku, slope_angle(num, rho2 + dot), fr);
+            const float t2 = fmaf(V.Ku, slope_angle(-num, rho2 - dot), fr);
+            lo[p] = fminf(t1, t2);
+            hi[p] = fmaxf(t1, t2);
+        }
+    } else {
+        const float r = cu * rcp_newton(cn);
+        split_cell(fmaf(V.Ku, r, V.Cu), aref, fr);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const float num = V.Ku * fmaf(-r, pn[p], pu[p]);
+            const float t1 = fr + __fdividef(num, cn + pn[p]);
+            const float t2 = fr - __fdividef(num, cn - pn[p]);
+            lo[p] = fminf(t1, t2);
+            hi[p] = fmaxf(t1, t2);
+        }
+    }
+    if (DD) {
+        k[0] = k[1] = lo[0];
+        k[2] = k[3] = hi[0];
+    } else {
+        k[0] = fminf(lo[0], lo[1]);
+        k[1] = fmaxf(lo[0], lo[1]);
+        k[2] = fminf(hi[0], hi[1]);
+        k[3] = fmaxf(hi[0], hi[1]);
+    }
+}
+
 // DD path length of cell (a, b): slab width times |d| / |d_main| of the ray
 // from the source to the cell centre (d in world coordinates).
 template <bool CURVED>

@@ -8,6 +8,15 @@
 
 namespace ctp {
 
+// Blocks of a cluster (at most 8, the portable size) that share a back's views:
+// as many as give the chip two waves of resident warps, while every block keeps
+// at least two of the npass rounds of views.  Depends on the geometry only.
+inline int view_split(long long warps, int npass) {
+    int s = 1;
+    while (s < 8 && warps * s < 2LL * 152 * 32 && npass >= 4 * s) s *= 2;
+    return s;
+}
+
 cudaError_t launch_sf(int dir, const CtGrid &g, const CtView *views, int in_t, const void *in,
                       int out_t, void *out, int batch, cudaStream_t st);
 cudaError_t launch_dd(int dir, const CtGrid &g, const CtView *views, int in_t, const void *in,
@@ -38,7 +47,21 @@ enum FanKind { FAN_SF = 0, FAN_DD = 1, FAN_TT = 2, FAN_VOX = 3, FAN_RAY = 4 };
 bool fan_fits(const CtGrid &g, int kind, int dir);
 cudaError_t launch_fan(int kind, int dir, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                        void *out, int batch, cudaStream_t st);
-// voxel-driven forward in circular geometry (the streaming forward of k_sf.cu)
+// circular cone-beam back (k_circ_back.cuh) of SF-TR, DD (from the scaled FP32
+// sinogram) and voxel-driven, recon: in recon mode; for footprints of at most
+// 8 cells and voxels shorter than 8 rows on a detector of at least 8 cells
+enum BackKind { BK_SF = 0, BK_DD = 1, BK_VOX = 2 };
+bool circ_back_fits(const CtGrid &g, int kind);
+cudaError_t launch_circ_back(int kind, bool recon, const CtGrid &g, const CtView *views, int in_t, const void *in,
+                             int out_t, void *out, int batch, cudaStream_t st);
+// circular cone-beam forward (k_circ_fwd.cuh) of SF-TR, DD and voxel-driven
+// (kind: BackKind) for footprints of at most 8 cells; cudaErrorMemoryAllocation
+// when its copies of the volume (circ_fwd_workspace bytes) cannot be had
+size_t circ_fwd_workspace(const CtGrid &g, int batch, int elem_bytes);
+bool circ_fwd_fits(const CtGrid &g, int kind, int batch);
+cudaError_t launch_circ_fwd(int kind, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
+                            void *out, int batch, cudaStream_t st);
+// voxel-driven forward in circular geometry (that kernel, or k_sf.cu without the copy)
 cudaError_t launch_vx_fwd_circ(const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                                void *out, int batch, cudaStream_t st);
 // recon mode (FBP): the pre-weighted ramp filter of each detector row, and the
@@ -61,9 +84,18 @@ cudaError_t launch_ray(int dir, const CtGrid &g, const CtView *views, int in_t, 
 cudaError_t launch_dd_back_scratch(const CtGrid &g, const CtView *views, int in_t, const void *in,
                                    int out_t, void *out, int batch, float *scratch, cudaStream_t st);
 
-// xZ[b][j][i][k] = x[b][k][j][i] for elements of elem_bytes (2 or 4) bytes
-cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny, int nz, int batch,
+// xZ[b][j][i][k] = x[b][k][j][i] for elements of elem_bytes (2 or 4) bytes,
+// columns nzp elements apart, zero from nz on
+cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny, int nz, int nzp, int batch,
                         cudaStream_t st);
+// slices of the circular forwards' copies of the volume: nz rounded up to four,
+// or 0: no copy (fan beam, non-circular, and volumes of fewer than four slices,
+// which the padding would double and more)
+inline int zmajor_pitch(const CtGrid &g) {
+    return g.is2d || g.variant == GEO_NONCIRC_FLAT || g.nz < 4 ? 0 : (g.nz + 3) & ~3;
+}
+// the copy's grid (rows and batch items are its y and z)
+inline bool zmajor_copy_fits(const CtGrid &g, int batch) { return batch <= 65535 && g.ny <= 65535; }
 
 // Stream-ordered scratch from a library-owned pool on the current device
 // (memory is kept in the pool between calls, so steady-state calls do not

@@ -242,7 +242,7 @@ template <typename TIn, int KIND, int NA, int NB> struct NcFwd {
         if (workspace_alloc((void **)&xZ, n * sizeof(TIn), st) != cudaSuccess) {
             cudaGetLastError();
             xZ = nullptr;
-        } else if ((e = zmajor_copy(sizeof(TIn), src, xZ, g.nx, g.ny, g.nz, batch, st)) != cudaSuccess) {
+        } else if ((e = zmajor_copy(sizeof(TIn), src, xZ, g.nx, g.ny, g.nz, g.nz, batch, st)) != cudaSuccess) {
             workspace_free(xZ, st);
             return e;
         }

@@ -560,9 +560,8 @@ template <int RPT, int NA> struct SfFwdSmem {
 // between cells floor(fu), floor(fu) + 1 with hat weights, and each voxel's
 // centre between rows floor(fv), floor(fv) + 1; Z accumulates amp x hat x.
 template <typename TIn, bool CURVED, int BV, int NA>
-__device__ __forceinline__ void vx_stage1(const CtView &V, const CtGrid &g, int i, int j, int B0, int bt,
-                                          const TIn *__restrict__ x, const TIn *__restrict__ volZ,
-                                          float (&Z)[BV][kItems], float (&Fu)[NA][kItems + 8], int *a0, int tid) {
+__device__ __forceinline__ void vx_stage1(const CtView &V, const CtGrid &g, int i, int j, int B0,
+                                          const TIn *__restrict__ x, float (&Z)[BV][kItems], float (&Fu)[NA][kItems + 8], int *a0, int tid) {
     const VxCol C = vx_col<CURVED>(V, g, i, j);
     const float af = floorf(C.fu), ta = C.fu - af;
     Fu[0][tid] = 1.f - ta;
@@ -587,21 +586,10 @@ __device__ __forceinline__ void vx_stage1(const CtView &V, const CtGrid &g, int 
         if (r0 >= 0 && r0 < BV) Z[r0][tid] = fmaf(1.f - tb, val, Z[r0][tid]);
         if (r0 + 1 >= 0 && r0 + 1 < BV) Z[r0 + 1][tid] = fmaf(tb, val, Z[r0 + 1][tid]);
     };
-    if (volZ != nullptr) {  // contiguous column of the z-major copy, 4 voxels per load
-        const TIn *cz = volZ + (size_t)bt * g.nx * g.ny * g.nz + ((size_t)j * g.nx + i) * g.nz;
-        for (int kq = k0 & ~3; kq <= k1; kq += 4) {
-            float xv[4];
-            ld4(cz + kq, xv);
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (kq + t >= k0 && kq + t <= k1) tap(kq + t, xv[t]);
-        }
-    } else {
-        const TIn *xc = x + (size_t)j * g.nx + i;
-        const size_t zs = (size_t)g.nx * g.ny;
+    const TIn *xc = x + (size_t)j * g.nx + i;
+    const size_t zs = (size_t)g.nx * g.ny;
 #pragma unroll 4
-        for (int k = k0; k <= k1; ++k) tap(k, ld(xc, (size_t)k * zs));
-    }
+    for (int k = k0; k <= k1; ++k) tap(k, ld(xc, (size_t)k * zs));
 }
 
 // SF-TT stage 1 of the streaming forward (flat detector): the column's
@@ -609,7 +597,7 @@ __device__ __forceinline__ void vx_stage1(const CtView &V, const CtGrid &g, int 
 // rows of its axial trapezoid (amplitude 1: A2 is applied per cell).
 template <typename TIn, int BV>
 __device__ __forceinline__ void tt_stage1(const CtView &V, const CtGrid &g, const SfCol &C, int i, int j, int B0,
-                                          int bt, const TIn *__restrict__ x, const TIn *__restrict__ volZ,
+                                          int bt, const TIn *__restrict__ x, const TIn *__restrict__ volZ, int nzp,
                                           float (&Z)[BV][kItems], int tid) {
     const TtCol T = tt_col(V, g, C, i, j);
     // voxels with a knot within a row of the tile (knots lie within the
@@ -631,7 +619,7 @@ __device__ __forceinline__ void tt_stage1(const CtView &V, const CtGrid &g, cons
             if (r0 + q >= 0 && r0 + q < BV) Z[r0 + q][tid] = fmaf(Fv[q], xv, Z[r0 + q][tid]);
     };
     if (volZ != nullptr) {  // contiguous column of the z-major copy, 4 voxels per load
-        const TIn *cz = volZ + (size_t)bt * g.nx * g.ny * g.nz + ((size_t)j * g.nx + i) * g.nz;
+        const TIn *cz = volZ + ((size_t)bt * g.nx * g.ny + (size_t)j * g.nx + i) * nzp;
 #pragma unroll 1
         for (int kq = k0 & ~3; kq <= k1; kq += 4) {
             float xv[4];
@@ -648,100 +636,13 @@ __device__ __forceinline__ void tt_stage1(const CtView &V, const CtGrid &g, cons
     }
 }
 
-// Axial sweep of one column in circular geometry (SF-TR or DD, axial
-// rectangle narrower than a row).  Voxel k covers rows [p_k - hv, p_k + hv]
-// with p_k = sv k + fv0 and sv = 2 hv, so consecutive rectangles abut: the
-// column's axial profile is a step function (value amp x on each voxel's
-// rectangle) and Z(row) is its integral over the row.  Walking k upward, a
-// voxel either lies inside the current row (adds w val, w = sv) or crosses
-// its upper edge once: the part below closes the row, whose sum is stored
-// once, and the rest opens the next.  d is the distance from the voxel's
-// lower edge to that row edge.  The walk runs over whole groups of four
-// voxels from k0 & ~3 (k0 & ~7 when nz is a multiple of 8) to k1 | 3 of the
-// z-major column (nz a multiple of 4); voxels outside [k0, k1] reach only
-// rows outside the tile, whose sums are dropped.  Rows the walk does not
-// reach are zero.
-template <typename TIn, bool DD, int BV>
-__device__ __forceinline__ void sf_sweep(const SfCol &C, const CtGrid &g, const CtView &V,
-                                         const TIn *__restrict__ cz, int k0, int k1, int B0,
-                                         float (&Z)[BV][kItems], int tid) {
-    // groups of eight from a sector boundary when nz is a multiple of 8
-    const int ks = (g.nz & 7) ? (k0 & ~3) : (k0 & ~7), ke = k1 | 3;
-    const float w = C.sv;
-    int bref;
-    float frac;
-    split_cell(fmaf(C.sv, (float)ks, C.fv0), bref, frac);
-    const float lo = frac - C.hv;  // lower edge, rows from bref: [-1, 0.5)
-    const int e0 = lo < -0.5f ? -1 : 0;
-    int r = bref + e0 - B0;          // tile row holding the lower edge
-    float d = ((float)e0 + 0.5f) - lo;  // to that row's upper edge: (0, 1]
-    const int rfirst = r;
-    float acc = 0.f;
-    const float wz0 = fmaf((float)ks, g.dz, V.o[2]);
-    // amplitude x value of voxels ks + t, ks + t + 1, in packed FP32x2
-    auto vals = [&](int t, float x0, float x1) {
-        if (DD) return make_float2(x0, x1);
-        const float2 wz2 = make_float2(fmaf((float)t, g.dz, wz0), fmaf((float)(t + 1), g.dz, wz0));
-        const float2 q = __ffma2_rn(wz2, wz2, make_float2(C.rxy2, C.rxy2));
-        const float2 amp = __fmul2_rn(__fmul2_rn(make_float2(C.invm, C.invm), q), make_float2(rsqrtf(q.x), rsqrtf(q.y)));
-        return __fmul2_rn(amp, make_float2(x0, x1));
-    };
-    auto step = [&](float val) {
-        const bool cross = d < w;
-        const float sum = fmaf(cross ? d : w, val, acc);
-        const float rest = (w - d) * val;
-        if (cross && (unsigned)r < (unsigned)BV) Z[r][tid] = sum;
-        acc = cross ? rest : sum;
-        r += cross ? 1 : 0;
-        d = (cross ? d + 1.f : d) - w;
-    };
-    // eight voxels (one 32-byte sector of FP32) per iteration
-    int kq = ks;
-    if ((g.nz & 7) == 0) {  // groups start on 8-element boundaries: one vector load each
-        for (; kq + 7 <= ke; kq += 8) {
-            float x8[8];
-            ld8(cz + kq, x8);
-#pragma unroll
-            for (int t = 0; t < 8; t += 2) {
-                const float2 v2 = vals(kq - ks + t, x8[t], x8[t + 1]);
-                step(v2.x);
-                step(v2.y);
-            }
-        }
-    }
-    for (; kq + 7 <= ke; kq += 8) {
-        float x8[8];
-        ld4(cz + kq, x8);
-        ld4(cz + kq + 4, x8 + 4);
-#pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-            const float2 v2 = vals(kq - ks + t, x8[t], x8[t + 1]);
-            step(v2.x);
-            step(v2.y);
-        }
-    }
-    if (kq <= ke) {
-        float xa[4];
-        ld4(cz + kq, xa);
-#pragma unroll
-        for (int t = 0; t < 4; t += 2) {
-            const float2 v2 = vals(kq - ks + t, xa[t], xa[t + 1]);
-            step(v2.x);
-            step(v2.y);
-        }
-    }
-    if ((unsigned)r < (unsigned)BV) Z[r][tid] = acc;
-    for (int q = 0; q < min(rfirst, BV); ++q) Z[q][tid] = 0.f;
-    for (int q = max(r + 1, 0); q < BV; ++q) Z[q][tid] = 0.f;
-}
-
 // (with up to 4 cells per item the SF-TR, DD and voxel-driven kernels fit 80
 // registers: 3 blocks per SM)
 // TT: SF-TT (flat detector); the per-cell amplitude A2 is applied after the gather.
 template <typename TIn, bool CURVED, bool DD, int RPT, int NA, bool VOX = false, bool TT = false>
 __global__ void __launch_bounds__(256, (NA <= 4 && !TT) ? 3 : 2)
 sf_fwd_circ(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
-            const TIn *__restrict__ volZ, void *__restrict__ sino, int out_t, int tiles_u, int tiles_v) {
+            const TIn *__restrict__ volZ, int nzp, void *__restrict__ sino, int out_t, int tiles_u, int tiles_v) {
     constexpr int BV = 8 * RPT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SfFwdSmem<RPT, NA> &S = *reinterpret_cast<SfFwdSmem<RPT, NA> *>(smem_raw);
@@ -805,7 +706,7 @@ sf_fwd_circ(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const int i = main_y ? l : s, j = main_y ? s : l;
                 const int sl = tid;  // this item's slot in the shared arrays
                 if constexpr (VOX) {
-                    vx_stage1<TIn, CURVED, BV, NA>(V, g, i, j, B0, bt, x, volZ, S.Z, S.Fu, S.a0, sl);
+                    vx_stage1<TIn, CURVED, BV, NA>(V, g, i, j, B0, x, S.Z, S.Fu, S.a0, sl);
                 } else {
                 const SfCol C = sf_col<CURVED, DD>(V, g, i, j);
                 int d0 = (int)floorf(C.T.k0 + 0.5f), d1 = (int)floorf(C.T.k3 + 0.5f);
@@ -821,16 +722,10 @@ sf_fwd_circ(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const float kb = ((float)(B0 + BV - 1) - C.fv0 + hw) * rsv;
                 const int k0 = max(0, (int)ceilf(fminf(ka, kb)));
                 const int k1 = min(g.nz - 1, (int)floorf(fmaxf(ka, kb)));
-                if (!TT && C.hv < 0.5f && C.sv > 0.f && volZ != nullptr && k0 <= k1) {
-                    // axial rectangle shorter than a row, column contiguous in
-                    // the z-major copy (nz a multiple of 4): one sweep down z
-                    const TIn *cz = volZ + (size_t)bt * g.nx * g.ny * g.nz + ((size_t)j * g.nx + i) * g.nz;
-                    sf_sweep<TIn, DD, BV>(C, g, V, cz, k0, k1, B0, S.Z, sl);
-                } else {
 #pragma unroll
                 for (int r = 0; r < BV; ++r) S.Z[r][sl] = 0.f;
                 if constexpr (TT) {
-                    tt_stage1<TIn, BV>(V, g, C, i, j, B0, bt, x, volZ, S.Z, sl);
+                    tt_stage1<TIn, BV>(V, g, C, i, j, B0, bt, x, volZ, nzp, S.Z, sl);
                 } else {
                 const TIn *xc = x + (size_t)j * g.nx + i;
                 const size_t zs = (size_t)g.nx * g.ny;
@@ -864,7 +759,6 @@ sf_fwd_circ(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                                 S.Z[r][sl] = fmaf(overlap(vf - C.hv, vf + C.hv, e - 0.5f, e + 0.5f), val, S.Z[r][sl]);
                         }
                     }
-                }
                 }
                 }
                 }
@@ -1065,25 +959,26 @@ dd_prescale(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
 
 // ------------------------------------------------------------ z-major copy
 // xZ[b][j][i][k] = x[b][k][j][i]: each voxel column contiguous, for the
-// forward's column walks.  32 x 33 shared-memory tiles over (i, k).
+// forward's column walks, padded with zeros to nzp elements.  32 x 33
+// shared-memory tiles over (i, k).
 template <typename T>
 __global__ void __launch_bounds__(256)
-to_zmajor(const T *__restrict__ x, T *__restrict__ xZ, int nx, int ny, int nz) {
+to_zmajor(const T *__restrict__ x, T *__restrict__ xZ, int nx, int ny, int nz, int nzp) {
     __shared__ T tile[32][33];
     const int tiles_i = (nx + 31) / 32;
     const int i0 = (blockIdx.x % tiles_i) * 32, k0 = (blockIdx.x / tiles_i) * 32;
     const int j = blockIdx.y;
     const size_t nvox = (size_t)nx * ny * nz;
     const T *src = x + blockIdx.z * nvox;
-    T *dst = xZ + blockIdx.z * nvox;
+    T *dst = xZ + blockIdx.z * ((size_t)nx * ny * nzp);
     for (int r = threadIdx.y; r < 32; r += 8) {  // rows of k, coalesced along i
         const int k = k0 + r, i = i0 + threadIdx.x;
-        if (i < nx && k < nz) tile[r][threadIdx.x] = src[((size_t)k * ny + j) * nx + i];
+        if (i < nx && k < nzp) tile[r][threadIdx.x] = k < nz ? src[((size_t)k * ny + j) * nx + i] : T(0.f);
     }
     __syncthreads();
     for (int r = threadIdx.y; r < 32; r += 8) {  // rows of i, coalesced along k
         const int i = i0 + r, k = k0 + threadIdx.x;
-        if (i < nx && k < nz) dst[((size_t)j * nx + i) * nz + k] = tile[threadIdx.x][r];
+        if (i < nx && k < nzp) dst[((size_t)j * nx + i) * nzp + k] = tile[threadIdx.x][r];
     }
 }
 
@@ -1103,23 +998,23 @@ cudaError_t fp_fwd_stream(const CtGrid &g, const CtView *views, const TIn *src, 
     cudaError_t e = cudaFuncSetAttribute(sf_fwd_circ<TIn, CURVED, DD, RPT, NA, VOX, TT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // a z-major copy of the volume (pooled workspace) makes every column walk
-    // a contiguous, vector-loaded read; without it the walks read strided
+    // SF-TT walks a z-major copy of the volume (pooled workspace), one vector
+    // load per four voxels; without it, and in the other projectors (here only
+    // when that copy could not be had), the walks read strided
     TIn *xZ = nullptr;
-    if (g.nz % 4 == 0 && g.nz >= 8) {
-        const size_t n = (size_t)g.nx * g.ny * g.nz * batch;
-        if (workspace_alloc((void **)&xZ, n * sizeof(TIn), st) != cudaSuccess) {
+    const int nzp = TT && zmajor_copy_fits(g, batch) ? zmajor_pitch(g) : 0;
+    if (nzp) {
+        if (workspace_alloc((void **)&xZ, (size_t)g.nx * g.ny * nzp * batch * sizeof(TIn), st) != cudaSuccess) {
             cudaGetLastError();
             xZ = nullptr;
-        } else {
-            dim3 tb(32, 8), tg((unsigned)(((g.nx + 31) / 32) * ((g.nz + 31) / 32)), (unsigned)g.ny,
-                               (unsigned)batch);
-            to_zmajor<TIn><<<tg, tb, 0, st>>>(src, xZ, g.nx, g.ny, g.nz);
+        } else if ((e = zmajor_copy(sizeof(TIn), src, xZ, g.nx, g.ny, g.nz, nzp, batch, st)) != cudaSuccess) {
+            workspace_free(xZ, st);
+            return e;
         }
     }
     dim3 blk(32, 8), grd((unsigned)((size_t)tiles_u * tiles_v * g.nview * batch));
-    sf_fwd_circ<TIn, CURVED, DD, RPT, NA, VOX, TT><<<grd, blk, smem, st>>>(g, views, src, xZ, out, out_t, tiles_u,
-                                                                      tiles_v);
+    sf_fwd_circ<TIn, CURVED, DD, RPT, NA, VOX, TT><<<grd, blk, smem, st>>>(g, views, src, xZ, nzp, out, out_t,
+                                                                           tiles_u, tiles_v);
     e = cudaGetLastError();
     if (xZ) {
         const cudaError_t ef = workspace_free(xZ, st);
@@ -1188,6 +1083,7 @@ cudaError_t sf_launch_t(int dir, const CtGrid &g, const CtView *views, const voi
 cudaError_t dd_back_scaled(const CtGrid &g, const CtView *views, const float *yp, void *out, int out_t, int batch,
                            cudaStream_t st) {
     if (g.is2d) return launch_fan(FAN_DD, 1, g, views, 0, yp, out_t, out, batch, st);
+    if (circ_back_fits(g, BK_DD)) return launch_circ_back(BK_DD, false, g, views, 0, yp, out_t, out, batch, st);
     return g.variant == GEO_CIRC_CURVED ? fp_back_circ<float, true, true>(g, views, yp, out, out_t, batch, st)
                                         : fp_back_circ<float, false, true>(g, views, yp, out, out_t, batch, st);
 }
@@ -1310,6 +1206,8 @@ cudaError_t launch_recon_fp(int dd, const CtGrid &g, const CtView *views, int in
                             void *out, int batch, cudaStream_t st) {
     if (g.variant == GEO_NONCIRC_FLAT) return launch_nc_recon(dd, g, views, in_t, in, out_t, out, batch, st);
     if (g.is2d) return launch_fan(dd ? FAN_DD : FAN_SF, 2, g, views, in_t, in, out_t, out, batch, st);
+    if (circ_back_fits(g, dd ? BK_DD : BK_SF))
+        return launch_circ_back(dd ? BK_DD : BK_SF, true, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return recon_fp_t<float>(dd, g, views, in, out, out_t, batch, st);
     case 1: return recon_fp_t<__half>(dd, g, views, in, out, out_t, batch, st);
@@ -1317,18 +1215,24 @@ cudaError_t launch_recon_fp(int dd, const CtGrid &g, const CtView *views, int in
     }
 }
 
-cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny, int nz, int batch,
+cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny, int nz, int nzp, int batch,
                         cudaStream_t st) {
-    dim3 tb(32, 8), tg((unsigned)(((nx + 31) / 32) * ((nz + 31) / 32)), (unsigned)ny, (unsigned)batch);
+    dim3 tb(32, 8), tg((unsigned)(((nx + 31) / 32) * ((nzp + 31) / 32)), (unsigned)ny, (unsigned)batch);
     if (elem_bytes == 4)
-        to_zmajor<float><<<tg, tb, 0, st>>>(static_cast<const float *>(x), static_cast<float *>(xZ), nx, ny, nz);
+        to_zmajor<float><<<tg, tb, 0, st>>>(static_cast<const float *>(x), static_cast<float *>(xZ), nx, ny, nz, nzp);
     else
-        to_zmajor<__half><<<tg, tb, 0, st>>>(static_cast<const __half *>(x), static_cast<__half *>(xZ), nx, ny, nz);
+        to_zmajor<__half><<<tg, tb, 0, st>>>(static_cast<const __half *>(x), static_cast<__half *>(xZ), nx, ny, nz,
+                                             nzp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_vx_fwd_circ(const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                                void *out, int batch, cudaStream_t st) {
+    if (circ_fwd_fits(g, BK_VOX, batch)) {
+        const cudaError_t e = launch_circ_fwd(BK_VOX, g, views, in_t, in, out_t, out, batch, st);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+    }
     switch (in_t) {
     case 0: return vx_fwd_t<float>(g, views, in, out, out_t, batch, st);
     case 1: return vx_fwd_t<__half>(g, views, in, out, out_t, batch, st);
@@ -1370,6 +1274,13 @@ cudaError_t launch_sf(int dir, const CtGrid &g, const CtView *views, int in_t, c
     if (g.variant == GEO_NONCIRC_FLAT && nc_footprint_fits(g, 0))
         return launch_nc(0, dir, g, views, in_t, in, out_t, out, batch, st);
     if (fan_fits(g, FAN_SF, dir)) return launch_fan(FAN_SF, dir, g, views, in_t, in, out_t, out, batch, st);
+    if (dir == 0 && circ_fwd_fits(g, BK_SF, batch)) {
+        const cudaError_t e = launch_circ_fwd(BK_SF, g, views, in_t, in, out_t, out, batch, st);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+    }
+    if (dir == 1 && circ_back_fits(g, BK_SF))
+        return launch_circ_back(BK_SF, false, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return sf_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return sf_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);
@@ -1389,6 +1300,11 @@ cudaError_t launch_dd(int dir, const CtGrid &g, const CtView *views, int in_t, c
         }
     }
     if (dir == 0 && fan_fits(g, FAN_DD, 0)) return launch_fan(FAN_DD, 0, g, views, in_t, in, out_t, out, batch, st);
+    if (dir == 0 && circ_fwd_fits(g, BK_DD, batch)) {
+        const cudaError_t e = launch_circ_fwd(BK_DD, g, views, in_t, in, out_t, out, batch, st);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+    }
     switch (in_t) {
     case 0: return dd_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return dd_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);

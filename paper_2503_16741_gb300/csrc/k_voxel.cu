@@ -297,6 +297,7 @@ cudaError_t vx_recon_t(const CtGrid &g, const CtView *views, const void *in, voi
 cudaError_t launch_voxel_recon(const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                                void *out, int batch, cudaStream_t st) {
     if (g.is2d) return launch_fan(FAN_VOX, 2, g, views, in_t, in, out_t, out, batch, st);
+    if (circ_back_fits(g, BK_VOX)) return launch_circ_back(BK_VOX, true, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return vx_recon_t<float>(g, views, in, out, out_t, batch, st);
     case 1: return vx_recon_t<__half>(g, views, in, out, out_t, batch, st);
@@ -307,6 +308,8 @@ cudaError_t launch_voxel_recon(const CtGrid &g, const CtView *views, int in_t, c
 cudaError_t launch_voxel(int dir, const CtGrid &g, const CtView *views, int in_t, const void *in,
                          int out_t, void *out, int batch, cudaStream_t st) {
     if (g.is2d) return launch_fan(FAN_VOX, dir, g, views, in_t, in, out_t, out, batch, st);
+    if (dir == 1 && circ_back_fits(g, BK_VOX))
+        return launch_circ_back(BK_VOX, false, g, views, in_t, in, out_t, out, batch, st);
     if (dir == 0 && g.variant != GEO_NONCIRC_FLAT)
         return launch_vx_fwd_circ(g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {

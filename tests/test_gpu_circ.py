@@ -1,0 +1,96 @@
+"""The circular cone-beam projection pair over its dispatch: taps of a footprint
+(1 to 8 cells, and beyond), rows per voxel (below 1, 2, 4 and 8, and beyond),
+chunks, patches, tiles and columns with remainders, views split over a cluster
+and not, against the FP64 oracle at the FP32 path's bound."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+import workloads as W
+from gpu_util import TOL_F32, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ct():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_16741_gb300 as ct
+    ct.load()
+    return ct
+
+
+# nx, ny, nz, nu, nv, views, du, dv (voxels 1.6 x 1.6 x 1.3 mm, magnification about 2)
+SIZES = {
+    "narrow-short": (19, 13, 16, 40, 30, 12, 7.0, 3.1),      # 2 cells (DD), sv < 1, one chunk
+    "ragged": (17, 9, 37, 33, 47, 67, 3.4, 2.9),             # 3 / 4 cells, remainders, views split 8 ways
+    "tall": (9, 22, 21, 45, 35, 9, 2.4, 1.6),                # 4 / 8 cells, sv in (1, 2), no split
+    "taller": (10, 10, 45, 60, 70, 37, 1.3, 0.9),            # 8 cells, sv in (2, 4)
+    "tallest": (9, 9, 13, 70, 90, 21, 1.3, 0.5),             # 8 cells, sv in (4, 8)
+    "beyond": (6, 7, 5, 70, 60, 5, 0.7, 0.3),                # more than 8 cells, sv > 8: the general kernel
+    "narrow-detector": (12, 12, 12, 7, 20, 8, 3.0, 3.0),     # fewer cells than a window
+    "flat-volume": (12, 12, 3, 30, 40, 6, 2.6, 2.9),         # no z-major copy
+    "large-detector": (11, 10, 37, 290, 130, 3, 0.9, 1.1),   # tiles of 64 rows, and of 290 = 9 x 32 + 2 cells
+    "off": (24, 24, 140, 20, 40, 40, 2.2, 2.9),              # most of the volume beside the detector; 2 z-blocks
+}
+
+
+def _spec(det, nx, ny, nz, nu, nv, views, du, dv):
+    return W.GeometrySpec("circ3d", det, nx, ny, nz, 1.6, 1.6, 1.3, nu, nv, du, dv, views,
+                          theta=0.2 + 2 * np.pi * np.arange(views) / views, sad=320.0, sdd=640.0, x_src=1.2,
+                          z_src=-2.0, u_ofst=-2.6, v_ofst=1.7, x_ofst=2.0, y_ofst=-1.0, z_ofst=1.5)
+
+
+def _check(got, ref, what):
+    assert np.linalg.norm(ref) > 0
+    assert rel_l2(got, ref) <= TOL_F32, what
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+def test_circ_back_matches_oracle(ct, det, size, proj):
+    spec = _spec(det, *SIZES[size])
+    g = ct.Geometry.from_spec(spec)
+    y = W.random_sino(spec, seed=2, batch=2) - 0.3
+    yd = torch.as_tensor(y, dtype=torch.float32).cuda()
+    y = yd.double().cpu().numpy()  # the oracle's input is what the GPU was given
+    x, r = ct.back(g, yd, proj), ct.back(g, yd, proj, mode="recon")
+    for b in range(2):
+        _check(x[b].cpu().numpy(), oracle.back(spec, proj, y[b]), "proj")
+        _check(r[b].cpu().numpy(), oracle.back_recon(spec, y[b], proj), "recon")
+    assert torch.equal(x[1], ct.back(g, yd[1].contiguous(), proj))
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+def test_circ_forward_matches_oracle(ct, det, size, proj):
+    spec = _spec(det, *SIZES[size])
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=2, batch=2) - 0.3, dtype=torch.float32).cuda()
+    y = ct.forward(g, x, proj)
+    for b in range(2):
+        _check(y[b].cpu().numpy(), oracle.forward(spec, proj, x[b].double().cpu().numpy()), "forward")
+    assert torch.equal(y[1], ct.forward(g, x[1].contiguous(), proj))
+    views = [0, 2]
+    assert torch.equal(ct.forward(g.subset(views), x, proj), y[:, views])
+
+
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+def test_a_bad_cell_stays_where_its_rays_go(ct, proj):
+    """An infinite detector cell reaches only voxels whose footprint is near it."""
+    spec = _spec("flat", *SIZES["ragged"])
+    g = ct.Geometry.from_spec(spec)
+    y = torch.rand(g.sino_shape, device="cuda")
+    clean = ct.back(g, y, proj)
+    y[3, 40, 16] = float("inf")
+    bad = ct.back(g, y, proj)
+    ok = torch.isfinite(bad)
+    assert torch.equal(bad[ok], clean[ok])
+    mask = np.zeros(spec.sino_shape)
+    mask[3, 38:43, 12:21] = 1.0
+    assert not (~ok.cpu().numpy() & (oracle.back(spec, "sf", mask) == 0)).any()
