@@ -194,6 +194,7 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     g->du = d->du;
     g->dv = two_d ? 1.0 : d->dv;
     const bool curved = d->det == CT_DET_CURVED;
+    double min_v = 1e30;  // lower bound on a voxel's axial height (rows)
     g->host_views.resize(d->nview);
     const std::vector<double> dbeta = recon_dbetas(d, P);
 
@@ -287,6 +288,10 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
         V.m_sf_u = (float)bound(D / g->du, hx * std::fabs(eu.x) + hy * std::fabs(eu.y),
                                 hx * std::fabs(n.x) + hy * std::fabs(n.y), tu);
         V.m_sf_v = (float)bound(D / g->dv, hz * std::fabs(ev.z), hz * std::fabs(n.z), tv);
+        // the height 2 K |hz ev.z - t hz n.z| / (depth (1 - ..)) of the farthest voxel, seen at the widest ratio t,
+        // from its farthest transaxial corner
+        min_v = std::min(min_v, 0.999 * (2.0 * D / g->dv) * hz * (std::fabs(ev.z) - tv * std::fabs(n.z)) /
+                                    (bmax + hx * std::fabs(n.x) + hy * std::fabs(n.y)));
         // SF-TT: the z faces at the transaxial corners (a 2D row lies inside the
         // axial plateau, so its factor is 1 and the bound does not matter)
         V.m_tt_v = two_d ? 0.25f
@@ -316,6 +321,7 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     G.max_m_dd_u = 0.f;
     G.max_m_sf_v = 0.f;
     G.max_m_tt_v = 0.f;
+    G.min_v = (float)min_v;
     for (const CtView &V : g->host_views) {
         G.max_m_sf_u = std::max(G.max_m_sf_u, V.m_sf_u);
         G.max_m_dd_u = std::max(G.max_m_dd_u, V.m_dd_u);

@@ -57,6 +57,7 @@ struct CtGrid {
     float max_m_dd_u;  // largest per-view DD boundary bound (cells)
     float max_m_sf_v;  // largest per-view axial half-height bound (rows)
     float max_m_tt_v;  // largest per-view SF-TT axial bound (rows)
+    float min_v;       // lower bound on a voxel's axial height on the detector (rows)
     float alpha, beta; // output epilogue: out = alpha * result + beta * out
 };
 

@@ -125,7 +125,7 @@ __device__ __forceinline__ void back_context(const CtView &V, const CtGrid &g, i
     S.as[t] = as;
     if (NT > 4) {
         S.n[t] = n;
-        S.nw[t] = __reduce_max_sync(__activemask(), n);
+        S.nw[t] = __reduce_max_sync(~0u, n);  // (whole warps form contexts)
     }
 #pragma unroll
     for (int q = 0; q < NT; ++q) S.F[q][t] = F[q];

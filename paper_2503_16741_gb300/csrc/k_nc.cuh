@@ -77,10 +77,43 @@ __device__ __forceinline__ int nc_cells(const Trap &T, int d0, int d1, float (&F
     return ql + 1;
 }
 
-// Footprint of voxel (i, j, k) in view V.  The centre is projected with a
-// correctly rounded reciprocal; corner and end-point offsets are formed from
-// small differences, K (du - r dn) / (cn + dn) with r = cu / cn, where a fast
-// division's few ulp are ~1e-7 cell.
+// What a column (i, j) shares down z in view V: the detector-frame components
+// of its voxel k = 0, and SF-TR's amplitude factors.
+struct NcCol {
+    float cu, cn, cv;
+    float im, r2;  // amplitude = im sqrt(wz^2 + r2)
+};
+template <int KIND> __device__ __forceinline__ NcCol nc_col(const CtView &V, const CtGrid &g, int i, int j) {
+    const float fi = (float)i, fj = (float)j;
+    NcCol C;
+    C.cu = fmaf(V.au[0], fi, fmaf(V.au[1], fj, V.au[3]));
+    C.cn = fmaf(V.an[0], fi, fmaf(V.an[1], fj, V.an[3]));
+    C.cv = fmaf(V.av[0], fi, fmaf(V.av[1], fj, V.av[3]));
+    C.im = 1.f;
+    C.r2 = 0.f;
+    if (KIND == NC_SF) {
+        const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
+        C.r2 = fmaf(wx, wx, wy * wy);
+        C.im = __fdividef(g.dx, fmaxf(fabsf(wx), fabsf(wy)));
+    }
+    return C;
+}
+
+// The two points at +- (d, dn) from a centre at ratio r = c / cn, in cells from
+// position f: K (d - r dn) / (cn + dn) and its mirror image.  With x = dn / cn
+// both are s (-+ x +- 1) for one s = K rcn (d - r dn) / (1 - x^2), so a pair
+// costs one fast division and comes out ordered.
+__device__ __forceinline__ void nc_pair(float Krcn, float rcn, float r, float d, float dn, float f, float &lo, float &hi) {
+    const float x = dn * rcn;
+    const float s = __fdividef(Krcn * fmaf(-r, dn, d), fmaf(-x, x, 1.f));
+    const float base = fmaf(-s, x, f);
+    lo = base - fabsf(s);
+    hi = base + fabsf(s);
+}
+
+// Footprint of voxel k of column C in view V.  The centre is projected with a
+// reciprocal good to an ulp; corner and end-point offsets are formed from small
+// differences, where a fast division's few ulp are ~1e-7 cell.
 //   SF-TR: trapezoid from the four transaxial corners x rectangle from the
 //          z ends at the (x, y) centre, voxel amplitude;
 //   DD:    box between the lateral boundary points x the same rectangle;
@@ -90,35 +123,38 @@ __device__ __forceinline__ int nc_cells(const Trap &T, int d0, int d1, float (&F
 //          1e-7 of the voxel size counts as zero and takes the negative
 //          side), amplitude per cell.
 template <int KIND, int NA, int NB>
-__device__ __forceinline__ void nc_fp(const CtView &V, const CtGrid &g, int i, int j, int k, NcFp<NA, NB> &P) {
-    const float fi = (float)i, fj = (float)j, fk = (float)k;
-    const float cu = fmaf(V.au[0], fi, fmaf(V.au[1], fj, fmaf(V.au[2], fk, V.au[3])));
-    const float cn = fmaf(V.an[0], fi, fmaf(V.an[1], fj, fmaf(V.an[2], fk, V.an[3])));
-    const float cv = fmaf(V.av[0], fi, fmaf(V.av[1], fj, fmaf(V.av[2], fk, V.av[3])));
-    const float rcn = __frcp_rn(cn);
+__device__ __forceinline__ void nc_fp(const CtView &V, const CtGrid &g, const NcCol &C, float fk, NcFp<NA, NB> &P) {
+    const float cu = fmaf(V.au[2], fk, C.cu);
+    const float cn = fmaf(V.an[2], fk, C.cn);
+    const float cv = fmaf(V.av[2], fk, C.cv);
+    const float rcn = rcp_newton(cn);
     const float r = cu * rcn, rv = cv * rcn;
     int aref, bref;
     float fr, vr;
     split_cell(fmaf(V.Ku, r, V.Cu), aref, fr);
     split_cell(fmaf(V.Kv, rv, V.Cv), bref, vr);
+    const float Kur = V.Ku * rcn, Kvr = V.Kv * rcn;
     Trap T;
     if (KIND == NC_DD) {  // boundary points +- half a voxel along the lateral axis
         const int q = V.main_y ? 0 : 1;
-        const float hu = 0.5f * V.au[q], hn = 0.5f * V.an[q];
-        const float e1 = fr + V.Ku * __fdividef(fmaf(r, hn, -hu), cn - hn);
-        const float e2 = fr + V.Ku * __fdividef(fmaf(-r, hn, hu), cn + hn);
-        const float lo = fminf(e1, e2), hi = fmaxf(e1, e2);
-        T = nc_trap(lo, lo, hi, hi);
-    } else {  // the four transaxial corners, sorted into a trapezoid
-        float t0 = fr + V.Ku * __fdividef(fmaf(-r, V.cdn[0], V.cdu[0]), cn + V.cdn[0]);
-        float t1 = fr + V.Ku * __fdividef(fmaf(-r, V.cdn[1], V.cdu[1]), cn + V.cdn[1]);
-        float t2 = fr + V.Ku * __fdividef(fmaf(-r, V.cdn[2], V.cdu[2]), cn + V.cdn[2]);
-        float t3 = fr + V.Ku * __fdividef(fmaf(-r, V.cdn[3], V.cdu[3]), cn + V.cdn[3]);
-        sort4(t0, t1, t2, t3);
-        T = nc_trap(t0, t1, t2, t3);
+        float lo, hi;
+        nc_pair(Kur, rcn, r, 0.5f * V.au[q], 0.5f * V.an[q], fr, lo, hi);
+        T = Trap{lo, lo, hi, hi, 0.f, 0.f};
+    } else {  // the four transaxial corners: two pairs opposite about the centre
+        float l0, h0, l1, h1;
+        nc_pair(Kur, rcn, r, V.cdu[3], V.cdn[3], fr, l0, h0);
+        nc_pair(Kur, rcn, r, V.cdu[1], V.cdn[1], fr, l1, h1);
+        T = nc_trap(fminf(l0, l1), fmaxf(l0, l1), fminf(h0, h1), fmaxf(h0, h1));
     }
     const int d0 = (int)floorf(T.k0 + 0.5f), d1 = (int)floorf(T.k3 + 0.5f);
-    P.n = nc_cells<NA>(T, d0, d1, P.Fu);
+    if (KIND == NC_DD) {  // box: plain overlaps (zero past its last cell)
+#pragma unroll
+        for (int q = 0; q < NA; ++q)
+            P.Fu[q] = overlap(T.k0, T.k3, (float)(d0 + q) - 0.5f, (float)(d0 + q) + 0.5f);
+        P.n = min(d1 - d0 + 1, NA);
+    } else {
+        P.n = nc_cells<NA>(T, d0, d1, P.Fu);
+    }
     P.a0 = aref + d0;
     const float hzv = V.hzv, hzn = V.hzn;
     if (KIND == NC_TT) {
@@ -145,9 +181,8 @@ __device__ __forceinline__ void nc_fp(const CtView &V, const CtGrid &g, int i, i
             P.b0 = bref + e0;
         }
     } else {  // axial rectangle: the end points (z -+ dz/2) at the voxel's (x, y) centre
-        const float f1 = vr + V.Kv * __fdividef(fmaf(-rv, hzn, hzv), cn + hzn);
-        const float f2 = vr + V.Kv * __fdividef(fmaf(rv, hzn, -hzv), cn - hzn);
-        const float vlo = fminf(f1, f2), vhi = fmaxf(f1, f2);
+        float vlo, vhi;
+        nc_pair(Kvr, rcn, rv, hzv, hzn, vr, vlo, vhi);
         // overlaps with rows e0 .. e0 + NB - 1 (row e covers [e - 1/2, e + 1/2]);
         // vlo lies below the first row's upper edge m, so each later row's
         // overlap starts at its lower edge (equal to overlap() bit for bit)
@@ -166,10 +201,9 @@ __device__ __forceinline__ void nc_fp(const CtView &V, const CtGrid &g, int i, i
     if (KIND != NC_SF) {
         P.amp = 1.f;
     } else {
-        const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
         const float wz = fmaf(fk, g.dz, V.o[2]);
-        const float t = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
-        P.amp = __fdividef(g.dx * t * rsqrtf(t), fmaxf(fabsf(wx), fabsf(wy)));
+        const float t = fmaf(wz, wz, C.r2);
+        P.amp = C.im * t * rsqrtf(t);
     }
 }
 

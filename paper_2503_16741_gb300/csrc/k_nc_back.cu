@@ -1,29 +1,51 @@
 // k_nc_back.cu -- backprojection of the non-circular SF-TR and DD footprint
 // projectors and of SF-TT, and the entries for both directions (the
 // footprint and the dispatch are in k_nc.cuh).
+#include <cooperative_groups.h>
+
 #include "k_nc.cuh"
 
 namespace ctp {
 
 // ------------------------------------------------------------ back (gather)
-// Views staged per round: few enough that the sinogram rows a warp reads
-// for them stay in L1 while the thread runs over its voxels.
-constexpr int kNcViews = 16;
+constexpr int kNcViews = 8;  // views staged per round
 
-// Thread = voxel column (i, j) over ZT voxels; per round of views the thread
-// runs over its voxels one at a time (the per-voxel body appears once in the
-// code, which keeps the kernel within the instruction cache) with the
-// voxel's sum carried in shared memory between rounds.
+// rows b0 .. b0 + NB - 1 under the first NC of the footprint's weights
+template <typename TIn, int NC, int NA, int NB>
+__device__ __forceinline__ float nc_taps(const NcFp<NA, NB> &P, const TIn *__restrict__ yv, const CtGrid &g) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        const int b = P.b0 + q;
+        if (P.Fv[q] != 0.f && b >= 0 && b < g.nv) {
+            const TIn *row = yv + (size_t)b * g.nu + P.a0;
+            float rs = P.Fu[0] * ld(row, 0);
+#pragma unroll
+            for (int c = 1; c < NC; ++c) rs = fmaf(P.Fu[c], c < P.n ? ld(row, (size_t)c) : 0.f, rs);
+            s = fmaf(P.Fv[q], rs, s);
+        }
+    }
+    return s;
+}
+
+// Thread = voxel column (i, j) over ZT voxels; per view it forms what the
+// column shares and runs over its voxels one at a time (the per-voxel body
+// appears once in the code, which keeps the kernel within the instruction
+// cache) with the voxels' sums in shared memory.  Bound by instruction issue
+// (84 % of slots).  192^3 / 250 views FP16 SF-TR 19.8 -> 16.3 ms from forming
+// corner pairs with one division each and the column's share once per view;
+// 64^3 / 90 views DD 637 -> 280 us, the views split over a cluster besides.
 // RECON: the recon-mode (FBP) backprojection with the normalised footprint
 // as the interpolation: weight rc_w / depth^2 over the footprint's area x
 // height (SF-TR and DD).
 template <typename TIn, int KIND, int NA, int NB, int ZT, bool RECON = false>
 __global__ void __launch_bounds__(128, 8)
 nc_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino, void *__restrict__ vol,
-        int out_t, int tiles_x, int nzc) {
+        int out_t, int tiles_x, int nzc, int S) {
     __shared__ CtView sview[kNcViews];
     __shared__ float acc[ZT][128];
     int bx = blockIdx.x;
+    const int rank = bx % S; bx /= S;  // cluster rank: the block's share of the rounds of views
     const int tx = bx % tiles_x; bx /= tiles_x;
     const int kc = bx % nzc;
     const int bt = bx / nzc;
@@ -31,12 +53,12 @@ nc_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino
     const int j = blockIdx.y * 4 + threadIdx.y;
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const bool active = i < g.nx && j < g.ny;
-    const int kbeg = kc * ZT;
+    const int kbeg = kc * ZT, kend = min(kbeg + ZT, g.nz);
 #pragma unroll
     for (int q = 0; q < ZT; ++q) acc[q][tid] = 0.f;
     const size_t vstride = (size_t)g.nv * g.nu;
     const TIn *ys = sino + (size_t)bt * g.nview * vstride;
-    for (int v0 = 0; v0 < g.nview; v0 += kNcViews) {
+    for (int v0 = rank * kNcViews; v0 < g.nview; v0 += S * kNcViews) {
         const int nvc = min(kNcViews, g.nview - v0);
         __syncthreads();
         {
@@ -47,32 +69,24 @@ nc_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino
         }
         __syncthreads();
         if (!active) continue;
+        for (int vv = 0; vv < nvc; ++vv) {
+            const CtView &V = sview[vv];
+            const TIn *yv = ys + (size_t)(v0 + vv) * vstride;
+            const NcCol C = nc_col<KIND>(V, g, i, j);
 #pragma unroll 1
-        for (int kk = 0; kk < ZT; ++kk) {
-            const int k = kbeg + kk;
-            if (k >= g.nz) break;
-            float a = acc[kk][tid];
-            for (int vv = 0; vv < nvc; ++vv) {
-                const CtView &V = sview[vv];
-                const TIn *yv = ys + (size_t)(v0 + vv) * vstride;
+            for (int k = kbeg; k < kend; ++k) {
                 NcFp<NA, NB> P;
-                nc_fp<KIND, NA, NB>(V, g, i, j, k, P);
+                nc_fp<KIND, NA, NB>(V, g, C, (float)k, P);
                 float s = 0.f;
                 if (P.a0 >= 0 && P.a0 + NA <= g.nu) {
                     // the whole window on the detector: one row pointer and
-                    // predicated loads of the footprint's cells (no branches)
-#pragma unroll
-                    for (int q = 0; q < NB; ++q) {
-                        const int b = P.b0 + q;
-                        if (P.Fv[q] != 0.f && b >= 0 && b < g.nv) {
-                            const TIn *row = yv + (size_t)b * g.nu + P.a0;
-                            float rs = P.Fu[0] * ld(row, 0);
-#pragma unroll
-                            for (int c = 1; c < NA; ++c)
-                                rs = fmaf(P.Fu[c], c < P.n ? ld(row, (size_t)c) : 0.f, rs);
-                            s = fmaf(P.Fv[q], rs, s);
-                        }
-                    }
+                    // predicated loads of the footprint's cells (no branches);
+                    // the bound NA holds near the source, and most footprints
+                    // end by their fourth cell
+                    if (NA <= 4 || P.n <= 4)
+                        s = nc_taps<TIn, NA < 4 ? NA : 4, NA, NB>(P, yv, g);
+                    else
+                        s = nc_taps<TIn, NA, NA, NB>(P, yv, g);
                 } else {
                     // cells off the detector get weight 0 and a clamped
                     // (in-bounds) address; cells past the footprint are not read
@@ -100,30 +114,56 @@ nc_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino
                         }
                     }
                 }
+                float &a = acc[k - kbeg][tid];
                 a = fmaf(RECON ? V.rc_w / (P.cn * P.cn * P.size) : P.amp, s, a);
             }
-            acc[kk][tid] = a;
         }
     }
-    if (!active) return;
-    const size_t base = (size_t)bt * g.nz * g.ny * g.nx + (size_t)j * g.nx + i;
-#pragma unroll
-    for (int kk = 0; kk < ZT; ++kk) {
-        const int k = kbeg + kk;
-        if (k < g.nz) st_out(g, vol, base + (size_t)k * g.ny * g.nx, acc[kk][tid], out_t);
+    const size_t zs = (size_t)g.ny * g.nx;
+    const size_t base = ((size_t)bt * g.nz + kbeg) * zs + (size_t)j * g.nx + i;
+    if (S == 1) {
+        if (!active) return;
+        for (int kk = 0; kk < kend - kbeg; ++kk) st_out(g, vol, base + kk * zs, acc[kk][tid], out_t);
+        return;
     }
+    // the cluster's sums, in rank order: rank r stores the voxels r, r + S, ...
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    if (active)
+        for (int kk = rank; kk < kend - kbeg; kk += S) {
+            float s = 0.f;
+            for (int r = 0; r < S; ++r) s += cl.map_shared_rank(&acc[0][0], r)[kk * 128 + tid];
+            st_out(g, vol, base + kk * zs, s, out_t);
+        }
+    cl.sync();  // (a block's shared memory stays until all have read it)
 }
 
 namespace {
+// Small volumes split the views over the blocks of a cluster (see view_split).
+template <typename TIn, int KIND, int NA, int NB, bool RECON>
+cudaError_t nc_back_go(const CtGrid &g, const CtView *views, const void *in, void *out, int out_t, int batch,
+                       cudaStream_t st) {
+    constexpr int ZT = 8;
+    const int tiles_x = (g.nx + 31) / 32, nzc = (g.nz + ZT - 1) / ZT, tiles_y = (g.ny + 3) / 4;
+    const int S = view_split((long long)tiles_x * tiles_y * nzc * 4, (g.nview + kNcViews - 1) / kNcViews);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((size_t)S * tiles_x * nzc * batch), (unsigned)tiles_y);
+    cfg.blockDim = dim3(32, 4);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = S > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, nc_back<TIn, KIND, NA, NB, ZT, RECON>, g, views, static_cast<const TIn *>(in), out,
+                              out_t, tiles_x, nzc, S);
+}
+
 template <typename TIn, int KIND, int NA, int NB> struct NcBack {
     static cudaError_t go(const CtGrid &g, const CtView *views, const void *in, void *out, int out_t, int batch,
                           cudaStream_t st) {
-        constexpr int ZT = 8;
-        const int tiles_x = (g.nx + 31) / 32, nzc = (g.nz + ZT - 1) / ZT;
-        dim3 blk(32, 4), grd((unsigned)(tiles_x * nzc * batch), (unsigned)((g.ny + 3) / 4));
-        nc_back<TIn, KIND, NA, NB, ZT><<<grd, blk, 0, st>>>(g, views, static_cast<const TIn *>(in), out, out_t,
-                                                          tiles_x, nzc);
-        return cudaGetLastError();
+        return nc_back_go<TIn, KIND, NA, NB, false>(g, views, in, out, out_t, batch, st);
     }
 };
 }  // namespace
@@ -131,12 +171,7 @@ template <typename TIn, int KIND, int NA, int NB> struct NcBack {
 template <typename TIn, int KIND, int NA, int NB> struct NcBackRecon {
     static cudaError_t go(const CtGrid &g, const CtView *views, const void *in, void *out, int out_t, int batch,
                           cudaStream_t st) {
-        constexpr int ZT = 8;
-        const int tiles_x = (g.nx + 31) / 32, nzc = (g.nz + ZT - 1) / ZT;
-        dim3 blk(32, 4), grd((unsigned)(tiles_x * nzc * batch), (unsigned)((g.ny + 3) / 4));
-        nc_back<TIn, KIND, NA, NB, ZT, true><<<grd, blk, 0, st>>>(g, views, static_cast<const TIn *>(in), out,
-                                                                  out_t, tiles_x, nzc);
-        return cudaGetLastError();
+        return nc_back_go<TIn, KIND, NA, NB, true>(g, views, in, out, out_t, batch, st);
     }
 };
 
