@@ -27,9 +27,9 @@
  *     the sinogram scaled by each cell's path length, amplitude or secant,
  *     batch x nview x nv x nu floats (non-circular CT_DD only when its
  *     footprints fit the footprint kernels, at most 8 cells by 4 rows);
- *   ct_forward with CT_SF, CT_DD or CT_SF_TT (cone beam) and with CT_VOXEL
- *     (circular cone beam): a reordered copy of the volume, batch x nz x ny x
- *     nx elements of in_t; in circular geometry with nz rounded up to a
+ *   ct_forward with CT_SF, CT_DD, CT_SF_TT or CT_RAY (cone beam) and with
+ *     CT_VOXEL (circular cone beam): a reordered copy of the volume, batch x
+ *     nz x ny x nx elements of in_t; but for CT_RAY, in circular geometry with nz rounded up to a
  *     multiple of 4, twice that for CT_SF, CT_DD and CT_VOXEL, and none below 4
  *     slices (skipped, at some speed, when it cannot be had).
  * ct_workspace_bytes gives that size for a call; ct_workspace_limit caps

@@ -16,15 +16,19 @@
 //   ray:     the same blocks, thread = (ray, every eighth run of slabs).
 // Every sum has a fixed order that depends on the geometry only:
 // deterministic, and batch items do not depend on the batch.
+// Batch items go in pairs that share each footprint.
 // Measured against the circular kernels with nz = nv = 1 that served fan beam
 // before (forward + back of one pass): 128 x 128, 180 views, ray-driven
-// forward and voxel-driven back 310 -> 35 us; 512 x 512, 720 views, FBP
-// 2058 -> 514 us; 2 images of 301 x 301, 217 views, SF forward and back
-// 4460 -> 1192 us.
+// forward and voxel-driven back 310 -> 34 us; 512 x 512, 720 views, FBP
+// 2058 -> 436 us; 2 images of 301 x 301, 217 views, SF forward and back
+// 4460 -> 625 us (1192 us before the pairs and the cheaper footprint).
 #include <algorithm>
+#include <type_traits>
 
 #include "ct_device.cuh"
 #include "ct_launch.h"
+#include "k_nc.cuh"
+#include "k_ray.cuh"
 
 namespace ctp {
 
@@ -38,30 +42,31 @@ constexpr int kFanViews = 64;  // view records staged at a time
 template <int KIND, bool CURVED>
 __device__ __forceinline__ void fan_foot(const CtView &V, const CtGrid &g, int i, int j, float cu, float cn, Trap &T,
                                          int &aref, float &amp) {
-    float fr;
-    split_cell(Det<CURVED>::fu(V, cu, cn), aref, fr);
-    if (KIND == FAN_DD) {  // boundary points +- half a pixel along the non-main axis
-        const int q = V.main_y ? 0 : 1;
-        const float hu = 0.5f * V.au[q], hn = 0.5f * V.an[q];
-        const float e1 = fr + Det<CURVED>::dfu(V, cu, cn, -hu, -hn);
-        const float e2 = fr + Det<CURVED>::dfu(V, cu, cn, hu, hn);
-        T.k0 = T.k1 = fminf(e1, e2);
-        T.k2 = T.k3 = fmaxf(e1, e2);
-        T.h1 = T.h3 = 0.f;  // (unused: the box's weights are plain overlaps)
-        amp = 1.f;
+    float k[4];
+    column_knots<CURVED, KIND == FAN_DD>(V, cu, cn, aref, k);
+    amp = 1.f;
+    if (KIND == FAN_DD) {
+        T = Trap{k[0], k[0], k[3], k[3], 0.f, 0.f};  // (the box's weights are plain overlaps)
     } else {
-        float t0 = fr + Det<CURVED>::dfu(V, cu, cn, V.cdu[0], V.cdn[0]);
-        float t1 = fr + Det<CURVED>::dfu(V, cu, cn, V.cdu[1], V.cdn[1]);
-        float t2 = fr + Det<CURVED>::dfu(V, cu, cn, V.cdu[2], V.cdn[2]);
-        float t3 = fr + Det<CURVED>::dfu(V, cu, cn, V.cdu[3], V.cdn[3]);
-        sort4(t0, t1, t2, t3);
-        T = make_trap(t0, t1, t2, t3);
-        amp = 1.f;
+        T = nc_trap(k[0], k[1], k[2], k[3]);
         if (KIND == FAN_SF) {
             const float wx = fmaf((float)i, g.dx, V.o[0]), wy = fmaf((float)j, g.dy, V.o[1]);
             const float r2 = fmaf(wx, wx, wy * wy);
             amp = __fdividef(g.dx * r2 * rsqrtf(r2), fmaxf(fabsf(wx), fabsf(wy)));
         }
+    }
+}
+
+// u position (cells), and the squared depth of the voxel-driven and recon weights
+template <bool CURVED>
+__device__ __forceinline__ void fan_point(const CtView &V, float cu, float cn, float &fu, float &rden2) {
+    if (CURVED) {
+        fu = fmaf(V.Ku, atan2f(cu, cn), V.Cu);
+        rden2 = __fdividef(1.f, fmaf(cu, cu, cn * cn));
+    } else {
+        const float r = rcp_newton(cn);
+        fu = fmaf(V.Ku, cu * r, V.Cu);
+        rden2 = r * r;
     }
 }
 
@@ -88,43 +93,47 @@ __device__ __forceinline__ void fan_slab(float w, float e, float h, float &lo, f
 }
 
 // ------------------------------------------------------------ back (gather)
-// contribution of one view's row y to pixel (i, j)
-template <typename TIn, int KIND, bool CURVED, bool RECON>
-__device__ __forceinline__ float fan_back_view(const CtView &V, const CtGrid &g, const TIn *__restrict__ y, int i,
-                                               int j) {
+// adds one view's contributions to pixel (i, j) of NBT batch items, whose rows
+// y are ystride apart (the footprint is formed once for all of them)
+template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
+__device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, const TIn *__restrict__ y,
+                                              size_t ystride, int i, int j, float (&acc)[NBT]) {
     const float fi = (float)i, fj = (float)j;
     const float cu = fmaf(V.au[0], fi, fmaf(V.au[1], fj, V.au[3]));
     const float cn = fmaf(V.an[0], fi, fmaf(V.an[1], fj, V.an[3]));
     if (KIND == FAN_VOX) {
-        const float fu = Det<CURVED>::fu(V, cu, cn);
+        float fu, rden2;
+        fan_point<CURVED>(V, cu, cn, fu, rden2);
         const float af = floorf(fu), t = fu - af;
         const int a0 = (int)af;
         // cells off the detector weigh zero and read a clamped address
-        const float w0 = (a0 >= 0 && a0 < g.nu) ? 1.f - t : 0.f;
-        const float w1 = (a0 + 1 >= 0 && a0 + 1 < g.nu) ? t : 0.f;
-        const float r = fmaf(w1, ld(y, (size_t)min(max(a0 + 1, 0), g.nu - 1)),
-                             w0 * ld(y, (size_t)min(max(a0, 0), g.nu - 1)));
-        const float den2 = CURVED ? fmaf(cu, cu, cn * cn) : cn * cn;
-        if (RECON) return __fdividef(V.rc_w, den2) * r;
-        const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
-        const float r2 = fmaf(wx, wx, wy * wy);
-        return __fdividef((g.dx * g.dy / g.du) * V.D * r2 * rsqrtf(r2), den2) * r;
+        const float w0 = (unsigned)a0 < (unsigned)g.nu ? 1.f - t : 0.f;
+        const float w1 = (unsigned)(a0 + 1) < (unsigned)g.nu ? t : 0.f;
+        float amp = V.rc_w * rden2;
+        if (!RECON) {
+            const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
+            const float r2 = fmaf(wx, wx, wy * wy);
+            amp = (g.dx * g.dy / g.du) * V.D * r2 * rsqrtf(r2) * rden2;
+        }
+        const int c0 = min(max(a0, 0), g.nu - 1), c1 = min(max(a0 + 1, 0), g.nu - 1);
+#pragma unroll
+        for (int q = 0; q < NBT; ++q, y += ystride)
+            acc[q] = fmaf(amp, fmaf(w1, ld(y, (size_t)c1), w0 * ld(y, (size_t)c0)), acc[q]);
     } else if (KIND == FAN_RAY) {
         int aref;
+        float k[4];
+        column_knots<CURVED, false>(V, cu, cn, aref, k);  // the pixel's shadow
+        const int d0 = max((int)ceilf(k[0] - kSearchPad), -aref);
+        const int d1 = min((int)floorf(k[3] + kSearchPad), g.nu - 1 - aref);
+        if (d0 > d1) return;
+        float fu, unused;
+        fan_point<CURVED>(V, cu, cn, fu, unused);
+        int ref;
         float fr;
-        split_cell(Det<CURVED>::fu(V, cu, cn), aref, fr);
-        const float t0 = Det<CURVED>::dfu(V, cu, cn, V.cdu[0], V.cdn[0]);
-        const float t1 = Det<CURVED>::dfu(V, cu, cn, V.cdu[1], V.cdn[1]);
-        const float t2 = Det<CURVED>::dfu(V, cu, cn, V.cdu[2], V.cdn[2]);
-        const float t3 = Det<CURVED>::dfu(V, cu, cn, V.cdu[3], V.cdn[3]);
-        const float umin = fr + fminf(fminf(t0, t1), fminf(t2, t3));
-        const float umax = fr + fmaxf(fmaxf(t0, t1), fmaxf(t2, t3));
-        const int d0 = max((int)ceilf(umin - kSearchPad), -aref);
-        const int d1 = min((int)floorf(umax + kSearchPad), g.nu - 1 - aref);
+        split_cell(fu, ref, fr);  // (ref == aref: the same operations)
         const float rho = Det<CURVED>::den(cu, cn);
-        float s = 0.f;
         for (int d = d0; d <= d1; ++d) {
-            const float dfu = (float)d - fr;
+            const float dfu = (float)(d + (aref - ref)) - fr;
             float wx, wy, ex, ey;
             if (CURVED) {
                 float sg, cg;
@@ -147,9 +156,11 @@ __device__ __forceinline__ float fan_back_view(const CtView &V, const CtGrid &g,
             bool in = true;
             fan_slab(wx, ex, 0.5f * g.dx, lo, hi, in);
             fan_slab(wy, ey, 0.5f * g.dy, lo, hi, in);
-            if (in && hi > lo) s = fmaf(hi - lo, ld(y, (size_t)(aref + d)), s);
+            if (in && hi > lo) {
+#pragma unroll
+                for (int q = 0; q < NBT; ++q) acc[q] = fmaf(hi - lo, ld(y + q * ystride, (size_t)(aref + d)), acc[q]);
+            }
         }
-        return s;
     } else {
         Trap T;
         int aref;
@@ -157,10 +168,13 @@ __device__ __forceinline__ float fan_back_view(const CtView &V, const CtGrid &g,
         fan_foot<KIND, CURVED>(V, g, i, j, cu, cn, T, aref, amp);
         const int d0 = max((int)floorf(T.k0 + 0.5f), -aref);
         const int d1 = min((int)floorf(T.k3 + 0.5f), g.nu - 1 - aref);
-        float s = 0.f, Gp = fan_G<KIND>(T, (float)d0 - 0.5f);
+        float s[NBT], Gp = fan_G<KIND>(T, (float)d0 - 0.5f);
+#pragma unroll
+        for (int q = 0; q < NBT; ++q) s[q] = 0.f;
         for (int d = d0; d <= d1; ++d) {
             const float Gn = fan_G<KIND>(T, (float)d + 0.5f);
-            s = fmaf(Gn - Gp, ld(y, (size_t)(aref + d)), s);
+#pragma unroll
+            for (int q = 0; q < NBT; ++q) s[q] = fmaf(Gn - Gp, ld(y + q * ystride, (size_t)(aref + d)), s[q]);
             Gp = Gn;
         }
         if (RECON) {  // depth weight over the footprint's area (cells) x axial height (rows)
@@ -168,22 +182,26 @@ __device__ __forceinline__ float fan_back_view(const CtView &V, const CtGrid &g,
             const float area = 0.5f * ((T.k3 - T.k0) + (T.k2 - T.k1));
             amp = __fdividef(V.rc_w, den * V.Kv * fabsf(V.av[2]) * area);
         }
-        return amp * s;
+#pragma unroll
+        for (int q = 0; q < NBT; ++q) acc[q] = fmaf(amp, s[q], acc[q]);
     }
 }
 
-template <typename TIn, int KIND, bool CURVED, bool RECON>
+template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
 __global__ void __launch_bounds__(32 * kFanWarps)
 fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino, void *__restrict__ vol, int out_t,
          int tiles_x, int batch) {
     __shared__ CtView sview[kFanViews];
-    __shared__ float red[kFanWarps][32];
+    __shared__ float red[NBT][kFanWarps][32];
     const int lane = threadIdx.x, w = threadIdx.y, tid = w * 32 + lane;
     const int i = (int)(blockIdx.x % tiles_x) * 8 + (lane & 7), j = (int)(blockIdx.x / tiles_x) * 4 + (lane >> 3);
     const bool active = i < g.nx && j < g.ny;
-    for (int bt = blockIdx.y; bt < batch; bt += gridDim.y) {
-        const TIn *ys = sino + (size_t)bt * g.nview * g.nu;
-        float acc = 0.f;
+    const size_t ystride = (size_t)g.nview * g.nu;
+    for (int bt = blockIdx.y * NBT; bt < batch; bt += gridDim.y * NBT) {
+        const TIn *ys = sino + bt * ystride;
+        float acc[NBT];
+#pragma unroll
+        for (int q = 0; q < NBT; ++q) acc[q] = 0.f;
         for (int v0 = 0; v0 < g.nview; v0 += kFanViews) {
             const int n = min(kFanViews, g.nview - v0);
             __syncthreads();
@@ -193,15 +211,17 @@ fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sin
             __syncthreads();
             if (active)
                 for (int t = w; t < n; t += kFanWarps)
-                    acc += fan_back_view<TIn, KIND, CURVED, RECON>(sview[t], g, ys + (size_t)(v0 + t) * g.nu, i, j);
+                    fan_back_view<TIn, KIND, CURVED, RECON, NBT>(sview[t], g, ys + (size_t)(v0 + t) * g.nu,
+                                                                 ystride, i, j, acc);
         }
-        red[w][lane] = acc;
-        __syncthreads();
-        if (w == 0 && active) {
-            float s = red[0][lane];
 #pragma unroll
-            for (int q = 1; q < kFanWarps; ++q) s += red[q][lane];
-            st_out(g, vol, (size_t)bt * g.ny * g.nx + (size_t)j * g.nx + i, s, out_t);
+        for (int q = 0; q < NBT; ++q) red[q][w][lane] = acc[q];
+        __syncthreads();
+        if (w < NBT && active) {
+            float s = red[w][0][lane];
+#pragma unroll
+            for (int q = 1; q < kFanWarps; ++q) s += red[w][q][lane];
+            st_out(g, vol, (size_t)(bt + w) * g.ny * g.nx + (size_t)j * g.nx + i, s, out_t);
         }
     }
 }
@@ -212,19 +232,20 @@ fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sin
 // x amplitude x value into the warp's slice of shared memory), then each lane
 // adds, for its cell, the pixels between the two lines of constant u that
 // bound its footprint's reach (their lateral index is affine in the slab).
-template <typename TIn, int KIND, bool CURVED, int NA>
+template <typename TIn, int KIND, bool CURVED, int NA, int NBT>
 __global__ void __launch_bounds__(32 * kFanWarps)
 fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, void *__restrict__ sino, int out_t,
         int tiles_u) {
     __shared__ CtView V;
     __shared__ float Sw[kFanWarps][NA][32 + 1];
+    __shared__ float Sx[kFanWarps][NBT][32];
     __shared__ int Sa[kFanWarps][32];
-    __shared__ float red[kFanWarps][32];
+    __shared__ float red[NBT][kFanWarps][32];
     const int lane = threadIdx.x, w = threadIdx.y;
     int bx = blockIdx.x;
     const int tu = bx % tiles_u; bx /= tiles_u;
     const int v = bx % g.nview;
-    const int bt = bx / g.nview;
+    const int bt = bx / g.nview * NBT;
     if (w == 0 && lane < (int)(sizeof(CtView) / sizeof(float4)))
         reinterpret_cast<float4 *>(&V)[lane] = __ldg(reinterpret_cast<const float4 *>(views + v) + lane);
     __syncthreads();
@@ -237,8 +258,11 @@ fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
     const float q1 = 1.f / (c.ul - T1 * c.nl), q2 = 1.f / (c.ul - T2 * c.nl);
     const float p1 = fmaf(T1, c.n3, -c.u3) * q1, s1 = fmaf(T1, c.ns, -c.us) * q1;
     const float p2 = fmaf(T2, c.n3, -c.u3) * q2, s2 = fmaf(T2, c.ns, -c.us) * q2;
-    const TIn *x = vol + (size_t)bt * g.nx * g.ny;
-    float acc = 0.f;
+    const size_t npix = (size_t)g.nx * g.ny;
+    const TIn *x = vol + bt * npix;
+    float acc[NBT];
+#pragma unroll
+    for (int q = 0; q < NBT; ++q) acc[q] = 0.f;
     for (int s = w; s < nslab; s += kFanWarps) {
         const float fs = (float)s;
         const float la = fmaf(s1, fs, p1), lb = fmaf(s2, fs, p2);
@@ -251,17 +275,18 @@ fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
             const int l = base + lane;
             if (l <= L1) {
                 const int i = main_y ? l : s, j = main_y ? s : l;
-                const float xv = ld(x, (size_t)j * g.nx + i);
+#pragma unroll
+                for (int q = 0; q < NBT; ++q) Sx[w][q][lane] = ld(x + q * npix, (size_t)j * g.nx + i);
                 const float fi = (float)i, fj = (float)j;
                 const float cu = fmaf(V.au[0], fi, fmaf(V.au[1], fj, V.au[3]));
                 const float cn = fmaf(V.an[0], fi, fmaf(V.an[1], fj, V.an[3]));
                 if (KIND == FAN_VOX) {
-                    const float fu = Det<CURVED>::fu(V, cu, cn);
+                    float fu, rden2;
+                    fan_point<CURVED>(V, cu, cn, fu, rden2);
                     const float af = floorf(fu), t = fu - af;
                     const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
                     const float r2 = fmaf(wx, wx, wy * wy);
-                    const float den2 = CURVED ? fmaf(cu, cu, cn * cn) : cn * cn;
-                    const float val = __fdividef((g.dx * g.dy / g.du) * V.D * r2 * rsqrtf(r2), den2) * xv;
+                    const float val = (g.dx * g.dy / g.du) * V.D * r2 * rsqrtf(r2) * rden2;
                     Sw[w][0][lane] = (1.f - t) * val;
                     Sw[w][1][lane] = t * val;
                     Sa[w][lane] = (int)af;
@@ -270,15 +295,17 @@ fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
                     int aref;
                     float amp;
                     fan_foot<KIND, CURVED>(V, g, i, j, cu, cn, T, aref, amp);
-                    const int d0 = (int)floorf(T.k0 + 0.5f);
-                    const float val = amp * xv;
-                    float Gp = 0.f;
+                    const int d0 = (int)floorf(T.k0 + 0.5f), d1 = (int)floorf(T.k3 + 0.5f);
+                    float F[NA];
+                    if (KIND == FAN_DD) {
 #pragma unroll
-                    for (int q = 0; q < NA; ++q) {
-                        const float Gn = fan_G<KIND>(T, (float)(d0 + q) + 0.5f);
-                        Sw[w][q][lane] = (Gn - Gp) * val;
-                        Gp = Gn;
+                        for (int q = 0; q < NA; ++q)
+                            F[q] = overlap(T.k0, T.k3, (float)(d0 + q) - 0.5f, (float)(d0 + q) + 0.5f);
+                    } else {
+                        nc_cells<NA>(T, d0, d1, F);
                     }
+#pragma unroll
+                    for (int q = 0; q < NA; ++q) Sw[w][q][lane] = F[q] * amp;
                     Sa[w][lane] = aref + d0;
                 }
             }
@@ -286,26 +313,26 @@ fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
             const int cb = min(hi, min(base + 31, L1)) - base;
             for (int q = max(lo, base) - base; q <= cb; ++q) {
                 const int d = a - Sa[w][q];
-                if ((unsigned)d < (unsigned)NA) acc += Sw[w][d][q];
+                if ((unsigned)d < (unsigned)NA) {
+                    const float wt = Sw[w][d][q];
+#pragma unroll
+                    for (int e = 0; e < NBT; ++e) acc[e] = fmaf(wt, Sx[w][e][q], acc[e]);
+                }
             }
             __syncwarp();
         }
     }
-    red[w][lane] = acc;
-    __syncthreads();
-    if (w || a >= g.nu) return;
-    float s = red[0][lane];
 #pragma unroll
-    for (int q = 1; q < kFanWarps; ++q) s += red[q][lane];
-    st_out(g, sino, ((size_t)bt * g.nview + v) * g.nu + a, s * fan_cell_factor<KIND, CURVED>(V, g, a), out_t);
+    for (int e = 0; e < NBT; ++e) red[e][w][lane] = acc[e];
+    __syncthreads();
+    if (w >= NBT || a >= g.nu) return;
+    float s = red[w][0][lane];
+#pragma unroll
+    for (int q = 1; q < kFanWarps; ++q) s += red[w][q][lane];
+    st_out(g, sino, ((size_t)(bt + w) * g.nview + v) * g.nu + a, s * fan_cell_factor<KIND, CURVED>(V, g, a), out_t);
 }
 
-// Ray-driven forward: the chord lengths of Siddon's method taken slab by slab
-// along the ray's steeper axis (in pixels): the ray's lateral position is
-// affine in the slab and moves by at most one pixel across it, so a slab
-// meets one pixel, or two that split it at their common edge.  Thread = (ray,
-// run of slabs): no serial walk, every slab's loads independent, and the
-// sum scaled once by the length of the ray in one slab.
+// Ray-driven forward: thread = (ray, one of 8 runs of slabs), see ray_run.
 template <typename TIn, bool CURVED>
 __global__ void __launch_bounds__(32 * kFanWarps)
 fan_ray_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, void *__restrict__ sino,
@@ -317,104 +344,79 @@ fan_ray_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
     const int v = bx % g.nview;
     const int bt = bx / g.nview;
     const int a = tu * 32 + lane;
-    const CtView &V = views[v];
-    float cn_ = V.D, cu_ = g.du * ((float)a - V.Cu);
-    if (CURVED) {
-        float sg, cg;
-        sincosf(((float)a - V.Cu) / V.Ku, &sg, &cg);
-        cn_ = V.D * cg;
-        cu_ = V.D * sg;
-    }
-    const float d0 = fmaf(cn_, V.nn[0], cu_ * V.eu[0]), d1 = fmaf(cn_, V.nn[1], cu_ * V.eu[1]);
-    // source and direction in pixel units; pixel i spans [i - 1/2, i + 1/2)
-    const float X0 = -V.o[0] / g.dx, X1 = -V.o[1] / g.dy, D0 = d0 / g.dx, D1 = d1 / g.dy;
-    const bool my = fabsf(D1) >= fabsf(D0);  // slabs along y
-    const float Sm = my ? X1 : X0, So = my ? X0 : X1, Dm = my ? D1 : D0, Do = my ? D0 : D1;
-    const int nm = my ? g.ny : g.nx, no = my ? g.nx : g.ny;
-    const int sm = my ? g.nx : 1, so = my ? 1 : g.nx;  // strides of the slab and the lateral index
-    const float slope = Do / Dm;
-    const float inv = slope != 0.f ? 1.f / slope : 0.f;
-    // lateral position at the image's middle (with the slope's rounding taken
-    // back over the long way from the source), then slab by slab from there
-    const float mid = 0.5f * (float)(nm - 1);
-    const float way = mid - Sm;
-    const float yc = fmaf(way, slope, So) + way * (fmaf(-slope, Dm, Do) / Dm);
-    const TIn *x = vol + (size_t)bt * g.nx * g.ny;
-    const int per = (nm + kFanWarps - 1) / kFanWarps;
-    const int s0 = w * per, s1 = min(s0 + per, nm);
-    float acc = 0.f;
-    if (a < g.nu && s0 < s1) {
-        float y0 = fmaf((float)s0 - 0.5f - mid, slope, yc);
-        int j0 = (int)floorf(y0 + 0.5f);
-#pragma unroll 4
-        for (int s = s0; s < s1; ++s) {
-            const float y1 = fmaf((float)s + 0.5f - mid, slope, yc);
-            const int j1 = (int)floorf(y1 + 0.5f);
-            const TIn *row = x + (size_t)s * sm;
-            const float x0 = (unsigned)j0 < (unsigned)no ? ld(row, (size_t)j0 * so) : 0.f;
-            const float x1 = (j1 != j0 && (unsigned)j1 < (unsigned)no) ? ld(row, (size_t)j1 * so) : 0.f;
-            // share of the slab before the edge between them
-            const float f = j1 == j0 ? 1.f : fminf(fmaxf(((float)max(j0, j1) - 0.5f - y0) * inv, 0.f), 1.f);
-            acc = fmaf(f, x0, fmaf(1.f - f, x1, acc));
-            y0 = y1;
-            j0 = j1;
-        }
-    }
+    float acc = 0.f, len = 0.f;
+    if (a < g.nu)
+        acc = ray_run<TIn, CURVED, true, kFanWarps>(views[v], g, a, 0, vol + (size_t)bt * g.nx * g.ny, nullptr, w, len);
     red[w][lane] = acc;
     __syncthreads();
     if (w || a >= g.nu) return;
     float s = red[0][lane];
 #pragma unroll
     for (int q = 1; q < kFanWarps; ++q) s += red[q][lane];
-    s *= sqrtf(fmaf(d0, d0, d1 * d1)) / fabsf(Dm);
-    st_out(g, sino, ((size_t)bt * g.nview + v) * g.nu + a, s, out_t);
+    st_out(g, sino, ((size_t)bt * g.nview + v) * g.nu + a, s * len, out_t);
 }
 
 // ------------------------------------------------------------ launchers
 namespace {
-template <typename TIn, int KIND, bool CURVED>
+template <typename TIn, int KIND, bool CURVED, int NBT>
 cudaError_t fan_fwd_k(const CtGrid &g, const CtView *views, const TIn *src, void *out, int out_t, int batch,
                       cudaStream_t st) {
     const int tiles_u = (g.nu + 31) / 32;
-    dim3 blk(32, kFanWarps), grd((unsigned)((size_t)tiles_u * g.nview * batch));
+    dim3 blk(32, kFanWarps), grd((unsigned)((size_t)tiles_u * g.nview * (batch / NBT)));
     if constexpr (KIND == FAN_RAY) {
         fan_ray_fwd<TIn, CURVED><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
     } else if constexpr (KIND == FAN_VOX) {
-        fan_fwd<TIn, KIND, CURVED, 2><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
+        fan_fwd<TIn, KIND, CURVED, 2, NBT><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
     } else {
         // a footprint of half width m meets at most 4 cells when m <= 1.5, 8 when m <= 3.5
         const float m = KIND == FAN_DD ? g.max_m_dd_u : g.max_m_sf_u;
         if (m <= 1.5f)
-            fan_fwd<TIn, KIND, CURVED, 4><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
+            fan_fwd<TIn, KIND, CURVED, 4, NBT><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
         else
-            fan_fwd<TIn, KIND, CURVED, 8><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
+            fan_fwd<TIn, KIND, CURVED, 8, NBT><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_u);
     }
     return cudaGetLastError();
 }
 
-template <typename TIn, int KIND, bool CURVED, bool RECON>
+template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
 cudaError_t fan_back_k(const CtGrid &g, const CtView *views, const TIn *src, void *out, int out_t, int batch,
                        cudaStream_t st) {
     const int tiles_x = (g.nx + 7) / 8, tiles_y = (g.ny + 3) / 4;
-    dim3 blk(32, kFanWarps), grd((unsigned)tiles_x * (unsigned)tiles_y, (unsigned)std::min(batch, 65535));
-    fan_back<TIn, KIND, CURVED, RECON><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_x, batch);
+    dim3 blk(32, kFanWarps), grd((unsigned)tiles_x * (unsigned)tiles_y, (unsigned)std::min(batch / NBT, 65535));
+    fan_back<TIn, KIND, CURVED, RECON, NBT><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_x, batch);
     return cudaGetLastError();
+}
+
+// Batch items in pairs, which share each footprint, and the odd one alone (the
+// same operations on every item, so its result does not depend on its partner).
+template <typename TIn, int KIND, bool CURVED>
+cudaError_t fan_pairs(int dir, const CtGrid &g, const CtView *views, const TIn *src, void *out, int out_t, int batch,
+                      cudaStream_t st) {
+    const int two = KIND == FAN_RAY && dir == 0 ? 0 : batch & ~1;
+    const size_t nvol = (size_t)g.nx * g.ny, nsino = (size_t)g.nview * g.nu;
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto pair, const TIn *in, void *to, int n) {
+        constexpr int NBT = decltype(pair)::value ? 2 : 1;
+        if (dir == 0) return fan_fwd_k<TIn, KIND, CURVED, NBT>(g, views, in, to, out_t, n, st);
+        if constexpr (KIND == FAN_SF || KIND == FAN_DD || KIND == FAN_VOX)
+            if (dir == 2) return fan_back_k<TIn, KIND, CURVED, true, NBT>(g, views, in, to, out_t, n, st);
+        return fan_back_k<TIn, KIND, CURVED, false, NBT>(g, views, in, to, out_t, n, st);
+    };
+    if (two) e = go(std::true_type(), src, out, two);
+    if (e == cudaSuccess && batch > two) {
+        const size_t in_item = dir == 0 ? nvol : nsino, out_item = dir == 0 ? nsino : nvol;
+        e = go(std::false_type(), src + two * in_item,
+               static_cast<char *>(out) + two * out_item * (out_t == 0 ? 4 : 2), batch - two);
+    }
+    return e;
 }
 
 template <typename TIn, int KIND>
 cudaError_t fan_t(int dir, const CtGrid &g, const CtView *views, const void *in, void *out, int out_t, int batch,
                   cudaStream_t st) {
     const TIn *src = static_cast<const TIn *>(in);
-    const bool curved = g.variant == GEO_CIRC_CURVED;
-    if (dir == 0)
-        return curved ? fan_fwd_k<TIn, KIND, true>(g, views, src, out, out_t, batch, st)
-                      : fan_fwd_k<TIn, KIND, false>(g, views, src, out, out_t, batch, st);
-    if constexpr (KIND == FAN_SF || KIND == FAN_DD || KIND == FAN_VOX)
-        if (dir == 2)
-            return curved ? fan_back_k<TIn, KIND, true, true>(g, views, src, out, out_t, batch, st)
-                          : fan_back_k<TIn, KIND, false, true>(g, views, src, out, out_t, batch, st);
-    return curved ? fan_back_k<TIn, KIND, true, false>(g, views, src, out, out_t, batch, st)
-                  : fan_back_k<TIn, KIND, false, false>(g, views, src, out, out_t, batch, st);
+    return g.variant == GEO_CIRC_CURVED ? fan_pairs<TIn, KIND, true>(dir, g, views, src, out, out_t, batch, st)
+                                        : fan_pairs<TIn, KIND, false>(dir, g, views, src, out, out_t, batch, st);
 }
 
 template <typename TIn>
