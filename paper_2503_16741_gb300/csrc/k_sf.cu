@@ -111,11 +111,29 @@ __device__ __forceinline__ void tt_rows(const SfCol &C, const TtCol &T, float fk
                                         float (&Fv)[4]) {
     const float gk = fmaf(C.sv, fk, T.g0);
     const float cN = fmaf(gk, T.eN, vf), cF = fmaf(gk, T.eF, vf);
-    float t0 = cN - T.hN, t1 = cN + T.hN, t2 = cF - T.hF, t3 = cF + T.hF;
-    sort4(t0, t1, t2, t3);
-    const Trap Tv = nc_trap(t0, t1, t2, t3);
-    e0 = (int)floorf(Tv.k0 + 0.5f);
-    nc_cells<4>(Tv, e0, (int)floorf(Tv.k3 + 0.5f), Fv);
+    // each face pair is ordered, so lower and upper knots sort with min and max
+    const float l0 = cN - T.hN, l1 = cF - T.hF, u0 = cN + T.hN, u1 = cF + T.hF;
+    const float m0 = fmaxf(l0, l1), m1 = fminf(u0, u1);
+    const float k0 = fminf(l0, l1), k1 = fminf(m0, m1), k2 = fmaxf(m0, m1), k3 = fmaxf(u0, u1);
+    const float ef = floorf(k0 + 0.5f);
+    e0 = (int)ef;
+    // (evaluated as a general trapezoid, edge by edge with its own clamps: 96^3 /
+    // 120 views, two BF16 volumes, forward 1.59 -> 1.43 ms, back 1.18 -> 1.11 ms)
+    // antiderivative at the three inner row edges from the saturated ramps
+    // a = (u - k0) / (k1 - k0), b = (u - k2) / (k3 - k2): half their squares times
+    // the ramps' widths, plus what lies past them
+    const float wa = fmaxf(k1 - k0, 1e-30f), wb = fmaxf(k3 - k2, 1e-30f);
+    const float ia = __fdividef(1.f, wa), ib = __fdividef(1.f, wb), ha = 0.5f * wa, hb = 0.5f * wb;
+    float Gp = 0.f;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float u = ef + ((float)q + 0.5f);
+        const float a = __saturatef((u - k0) * ia), b = __saturatef((u - k2) * ib);
+        const float G = fmaf(a * a, ha, fmaxf(u - k1, 0.f)) - fmaf(b * b, hb, fmaxf(u - k3, 0.f));
+        Fv[q] = G - Gp;
+        Gp = G;
+    }
+    Fv[3] = fmaxf(0.5f * ((k3 - k0) + (k2 - k1)) - Gp, 0.f);
 }
 
 // the 4-cell window [as, as + 3] inside the detector (nu >= 4) for the weights
