@@ -2,7 +2,7 @@
 // projectors whose weight is transaxial x axial: SF-TR, DD and voxel-driven
 // (Sec. 2.3; Long, Fessler & Balter 2010; De Man & Basu 2004; Peters 1981).
 //
-// CTA = 32 detector cells x BV = 8 RPT rows of one view, 256 threads.  Work
+// CTA = 64 or 32 cells x BV = 64 or 32 rows of one view, 256 threads.  Work
 // items are the voxel columns (slab s, lateral l) whose footprint can reach the
 // tile, taken 256 at a time.
 //   stage 1: thread = item; it forms the column's transaxial weights (NT
@@ -26,11 +26,13 @@
 // cost a quarter of the kernel: 120 views of the 256^3 scan 5.5 -> 4.3 ms), and
 // the next four voxels are requested before the present ones are walked (the
 // curved scan below: 83 -> 50 ms, with three blocks per SM instead of two).
+// Of the 256^3 scan's time (11.4 ms before the 64-cell tiles), compiling parts
+// out left: set-up and search 1.3 ms, walk 5.6, stage 2 5.0.
 // Measured against the kernel before, 256^3 / 360 views / 512 x 384 FP32: SF-TR
-// 13.4 -> 11.8 ms, voxel-driven 19.2 -> 10.9 ms; 161^2 x 155 / 607 views, SF-TR
-// 10.4 -> 5.7 ms (no multiple of four slices); 183^2 x 157 / 231 views, DD with
+// 13.4 -> 10.7 ms, voxel-driven 19.2 -> 10.4 ms; 161^2 x 155 / 607 views, SF-TR
+// 10.4 -> 5.1 ms (no multiple of four slices); 183^2 x 157 / 231 views, DD with
 // voxels up to 1.2 rows high 6.4 -> 3.7 ms; curved 512^2 x 128 / 984 views, DD
-// 65.3 -> 49.7 ms.
+// 65.3 -> 48 ms.
 #pragma once
 #include <algorithm>
 
@@ -49,7 +51,7 @@ template <int BV, int NT> struct CircFwdSmem {
     // the item's transaxial weights x amplitude factor; rows padded by 8 so that
     // lanes reading one item's weights of different cells fall on different banks
     float Fu[NT][kFwdItems + 8];
-    short a0[kFwdItems];  // first cell of the item's weights, from the tile's first cell
+    short a0[kFwdItems + 2];  // first cell of the item's weights, from the tile's first cell
     unsigned short L0[kFwdSeg];  // first column of each slab (at most 65536 columns)
     int off[kFwdSeg + 1];        // first item of each slab
     int warp_sum[8];
@@ -64,8 +66,9 @@ template <int BV, int NT> struct CircFwdSmem {
 // two agree whatever the rounding.)  TALL: a voxel may cover whole rows.
 // Voxels outside [k0, k1] reach no row of the tile.
 template <typename TIn, int KIND, int BV, bool TALL>
-__device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict__ cz, size_t pitch, int k0, int k1, float sv,
-                                          float fv0, float r2, float oz, int B0, float (&Z)[BV][kFwdItems], int tid) {
+__device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict__ cz, size_t pitch, float (&xa)[4],
+                                          int k0, int k1, float sv, float fv0, float r2, float oz, int B0,
+                                          float (&Z)[BV][kFwdItems], int tid) {
     static_assert(kFwdItems * sizeof(float) == 1 << 10, "row stride of the walk");
     const int ks = k0 & ~3;
     float lo;  // of voxel ks
@@ -157,9 +160,9 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
         }
     };
     // four voxels per load, the next four requested before they are walked
+    // (xa: the first four, requested by the caller)
     const TIn *cq = cz + (size_t)(ks >> 2) * pitch;
-    float xa[4], xb[4];
-    ld4(cq, xa);
+    float xb[4];
     float kk = 0.f;
     for (int left = k1 - ks;; left -= 8, kk += 8.f) {
         if (left >= 4) ld4(cq + pitch, xb);
@@ -179,12 +182,13 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
     for (int q = max(r, 0); q < BV; ++q) Z[q][tid] = 0.f;
 }
 
-template <typename TIn, int KIND, bool CURVED, int RPT, int NT, bool TALL>
-// (BV = 64: 3 blocks per SM by shared memory and 80 registers; BV = 32: 4 at 64)
-__global__ void __launch_bounds__(256, RPT == 4 ? 4 : 3)
+// CTA = CELLS cells x BV rows, CELLS / 32 x NG warps, RPT rows to a thread.
+// (BV = 64: 3 blocks per SM by shared memory and 80 registers; 32 x 32: 4 at 64)
+template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL>
+__global__ void __launch_bounds__(256, BV == 32 ? 4 : 3)
 circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ volZ, int nzp, void *__restrict__ sino,
          int out_t, int tiles_u, int tiles_v) {
-    constexpr int BV = 8 * RPT;
+    constexpr int NG = 256 / CELLS, RPT = BV / NG;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CircFwdSmem<BV, NT> &S = *reinterpret_cast<CircFwdSmem<BV, NT> *>(smem_raw);
     int bx = blockIdx.x;
@@ -193,8 +197,10 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
     const int v = bx % g.nview;
     const int bt = bx / g.nview;
     const int tid = threadIdx.y * 32 + threadIdx.x;
-    const int A0 = tu * 32, B0 = tv * BV, Bn = min(BV, g.nv - B0);  // rows of the tile on the detector
-    const int a = A0 + threadIdx.x;
+    const int A0 = tu * CELLS, B0 = tv * BV, Bn = min(BV, g.nv - B0);  // rows of the tile on the detector
+    const int ac = (int)(threadIdx.y % (CELLS / 32)) * 32 + (int)threadIdx.x;  // the thread's cell in the tile
+    const int rg = (int)threadIdx.y / (CELLS / 32);                          // and its rows rg, rg + NG, ..
+    const int a = A0 + ac;
     const CtView &V = views[v];
     const int main_y = V.main_y;
     const SlabCoef sc = slab_coef(V, main_y);
@@ -225,7 +231,7 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
         int c = 0;
         if (tid < nseg) {
             int L0, L1, K0, K1;
-            if (slab_search<CURVED>(V, sc, seg + tid, A0 - mu, A0 + 31.f + mu, B0 - mv, B0 + Bn - 1.f + mv, nlat, g.nz,
+            if (slab_search<CURVED>(V, sc, seg + tid, A0 - mu, A0 + (CELLS - 1.f) + mu, B0 - mv, B0 + Bn - 1.f + mv, nlat, g.nz,
                                     L0, L1, K0, K1))
                 c = L1 - L0 + 1;
             S.L0[tid] = (unsigned short)(c ? L0 : 0);
@@ -245,19 +251,23 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
         }
         __syncthreads();
         const int total = S.off[nseg];
+        // last slab t' >= t with off[t'] <= q, by the whole warp: 32 offsets at a time
+        auto seek = [&](int t, int q) {
+            for (;;) {
+                const int u = t + 1 + (int)threadIdx.x;
+                const int c = __popc(__ballot_sync(~0u, u < nseg && S.off[min(u, nseg)] <= q));
+                t += c;
+                if (c < 32) return t;
+            }
+        };
+        int first = 0;  // slab of the round's first item
         for (int base = 0; base < total; base += kFwdItems) {
             // ---- stage 1: one item (column) per thread
             const int q = base + tid;
+            first = seek(first, base);
+            int lo = seek(first, base + (tid & ~31));  // slab of the warp's first item
             if (q < total) {
-                // slab of item q: last t with off[t] <= q.  The warp searches
-                // for its first item (every lane reads the same offsets), then
-                // each lane steps forward to its own (a slab holds tens of items)
-                const int qw = base + (tid & ~31);
-                int lo = 0, hi = nseg - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (S.off[mid] <= qw) lo = mid; else hi = mid - 1;
-                }
+                // each lane steps forward to its own item's slab (a slab holds tens of items)
                 while (lo < nseg - 1 && S.off[lo + 1] <= q) ++lo;
                 const int s = seg + lo;
                 const int l = S.L0[lo] + (q - S.off[lo]);
@@ -270,6 +280,15 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                 const float kd = V.Kv * rden;
                 const float sv = kd * V.av[2], fv0 = fmaf(kd, V.av[3], V.Cv);
                 const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
+                // voxels that can meet a row of the tile
+                const float hw = KIND == BK_VOX ? 1.f + kSearchPad : 0.5f + 0.5f * sv + kSearchPad;
+                const float rsv = __fdividef(1.f, sv);
+                const int k0 = max(0, (int)ceilf(((float)B0 - fv0 - hw) * rsv - 1e-3f));
+                const int k1 = min(g.nz - 1, (int)floorf(((float)(B0 + Bn - 1) - fv0 + hw) * rsv + 1e-3f));
+                const TIn *cz = xz + 4 * ((size_t)s * nlat + l);
+                const size_t pitch = 4 * (size_t)g.nx * g.ny;
+                float x4[4] = {0.f, 0.f, 0.f, 0.f};  // on its way while the weights are formed
+                if (k0 <= k1) ld4(cz + (size_t)(k0 >> 2) * pitch, x4);
                 if constexpr (KIND == BK_VOX) {
                     const float fu = CURVED ? fmaf(V.Ku, atan2f(cu, cn), V.Cu) : fmaf(V.Ku, cu * rden, V.Cu);
                     const float af = floorf(fu), amp = vx_amp(g, V, 1.f, CURVED ? den2 * rden : cn);
@@ -296,28 +315,18 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                     for (int r = 0; r < NT; ++r) S.Fu[r][tid] = F[r];
                     S.a0[tid] = (short)(aref + d0 - A0);
                 }
-                // voxels that can meet a row of the tile
-                const float hw = KIND == BK_VOX ? 1.f + kSearchPad : 0.5f + 0.5f * sv + kSearchPad;
-                const float rsv = __fdividef(1.f, sv);
-                const int k0 = max(0, (int)ceilf(((float)B0 - fv0 - hw) * rsv - 1e-3f));
-                const int k1 = min(g.nz - 1, (int)floorf(((float)(B0 + Bn - 1) - fv0 + hw) * rsv + 1e-3f));
                 if (k0 <= k1)
-                    circ_walk<TIn, KIND, BV, TALL>(g, xz + 4 * ((size_t)s * nlat + l), 4 * (size_t)g.nx * g.ny, k0, k1,
-                                                   sv, fv0, fmaf(wx, wx, wy * wy), V.o[2], B0, S.Z, tid);
+                    circ_walk<TIn, KIND, BV, TALL>(g, cz, pitch, x4, k0, k1, sv, fv0, fmaf(wx, wx, wy * wy), V.o[2], B0,
+                                                   S.Z, tid);
                 else
                     for (int r = 0; r < BV; ++r) S.Z[r][tid] = 0.f;
             }
             __syncthreads();
-            // ---- stage 2: thread = (cell a, rows B0 + threadIdx.y + 8 r)
+            // ---- stage 2: thread = (cell a, rows B0 + rg + NG r)
             if (a < g.nu) {
                 const int qend = min(total, base + kFwdItems);
-                int lo = 0, hi = nseg - 1;  // first slab with items in [base, qend)
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (S.off[mid] <= base) lo = mid; else hi = mid - 1;
-                }
-                const float *zr = &S.Z[threadIdx.y][0];
-                for (int t = lo, o0 = S.off[lo]; t < nseg && o0 < qend; ++t) {
+                const float *zr = &S.Z[rg][0];
+                for (int t = first, o0 = S.off[first]; t < nseg && o0 < qend; ++t) {
                     const int o1 = S.off[t + 1];
                     const float fs = (float)(seg + t);
                     const float la = fmaf(s1, fs, p1), lb = fmaf(s2, fs, p2);
@@ -326,8 +335,10 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                     const int c0 = max((int)ceilf(fminf(la, lb) - 1e-3f) + rel, max(o0 - base, 0));
                     const int c1 = min((int)floorf(fmaxf(la, lb) + 1e-3f) + rel, min(o1, qend) - base - 1);
                     o0 = o1;
-                    for (int c = c0; c <= c1; ++c) {
-                        const int d = (int)threadIdx.x - S.a0[c];
+                    if (c0 > c1) continue;
+                    for (int c = c0, next = S.a0[c0]; c <= c1; ++c) {
+                        const int d = ac - next;
+                        next = S.a0[c + 1];  // (the next item's, before this one's rows)
                         if ((unsigned)d >= (unsigned)NT) continue;
                         const float w = S.Fu[d][c];
                         const float *z = zr + c;
@@ -335,7 +346,7 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                             const float2 w2 = make_float2(w, w);
 #pragma unroll
                             for (int r = 0; r < RPT; r += 2)
-                                acc[r / 2] = __ffma2_rn(w2, make_float2(z[8 * r * kFwdItems], z[8 * (r + 1) * kFwdItems]),
+                                acc[r / 2] = __ffma2_rn(w2, make_float2(z[NG * r * kFwdItems], z[NG * (r + 1) * kFwdItems]),
                                                         acc[r / 2]);
                         } else {
                             acc[0].x = fmaf(w, z[0], acc[0].x);
@@ -349,7 +360,7 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
     if (a < g.nu) {
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
-            const int b = B0 + threadIdx.y + 8 * r;
+            const int b = B0 + rg + NG * r;
             const float s = (r & 1) ? acc[r / 2].y : acc[r / 2].x;
             if (b < g.nv)
                 st_out(g, sino, (((size_t)bt * g.nview + v) * g.nv + b) * g.nu + a,
@@ -360,12 +371,12 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
 
 // ------------------------------------------------------------ launchers
 namespace {
-template <typename TIn, int KIND, bool CURVED, int RPT, int NT, bool TALL>
+template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL>
 cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
                         cudaStream_t st) {
-    const int tiles_u = (g.nu + 31) / 32, tiles_v = (g.nv + 8 * RPT - 1) / (8 * RPT);
-    const size_t smem = sizeof(CircFwdSmem<8 * RPT, NT>);
-    auto kern = circ_fwd<TIn, KIND, CURVED, RPT, NT, TALL>;
+    const int tiles_u = (g.nu + CELLS - 1) / CELLS, tiles_v = (g.nv + BV - 1) / BV;
+    const size_t smem = sizeof(CircFwdSmem<BV, NT>);
+    auto kern = circ_fwd<TIn, KIND, CURVED, CELLS, BV, NT, TALL>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((unsigned)((size_t)tiles_u * tiles_v * g.nview * batch)), dim3(32, 8), smem, st>>>(
@@ -373,16 +384,20 @@ cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *xZ, int
     return cudaGetLastError();
 }
 
-// rows of a tile: 64, or 32 for a short detector and for a detector of few
-// tiles (more CTAs of a small scan); the choice does not depend on the views
-// or the batch, so a view's result does not either
+// Tiles of 64 cells x 64 rows, where a thread of stage 2 sums 16 rows and so
+// shares what it does per column among twice the rows of a 32 x 64 tile (256^3 /
+// 360 views SF-TR 11.4 -> 10.7 ms, 161^2 x 155 / 607 views 5.6 -> 5.1 ms); 32 x 64
+// where voxels may cover whole rows, whose walk takes the registers (64 x 64
+// spills: 183^2 x 157 / 231 views DD 3.7 -> 4.2 ms); 32 x 32 for a short detector
+// and for one of few tiles (more CTAs of a small scan).  The choice does not
+// depend on the views or the batch, so a view's result does not either.
 template <typename TIn, int KIND, bool CURVED, int NT, bool TALL>
 cudaError_t circ_fwd_rpt(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
                          cudaStream_t st) {
     const int tiles = ((g.nu + 31) / 32) * ((g.nv + 63) / 64);
     if (g.nv > 32 && tiles > 16)
-        return circ_fwd_go<TIn, KIND, CURVED, 8, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
-    return circ_fwd_go<TIn, KIND, CURVED, 4, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+        return circ_fwd_go<TIn, KIND, CURVED, TALL ? 32 : 64, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+    return circ_fwd_go<TIn, KIND, CURVED, 32, 32, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
 }
 
 template <typename TIn, int KIND, bool CURVED, int NT>
