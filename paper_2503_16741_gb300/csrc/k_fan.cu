@@ -20,7 +20,7 @@
 // Measured against the circular kernels with nz = nv = 1 that served fan beam
 // before (forward + back of one pass): 128 x 128, 180 views, ray-driven
 // forward and voxel-driven back 310 -> 34 us; 512 x 512, 720 views, FBP
-// 2058 -> 436 us; 2 images of 301 x 301, 217 views, SF forward and back
+// 2058 -> 383 us (436 us with one pixel to a thread); 2 images of 301 x 301, 217 views, SF forward and back
 // 4460 -> 625 us (1192 us before the pairs and the cheaper footprint).
 #include <algorithm>
 #include <type_traits>
@@ -187,21 +187,24 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
     }
 }
 
-template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
+// PX: pixels of a thread (the patch is 8 x 4 PX), which share the view record's
+// reads from shared memory: two in large images, where the warps suffice.
+template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT, int PX>
 __global__ void __launch_bounds__(32 * kFanWarps)
 fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino, void *__restrict__ vol, int out_t,
          int tiles_x, int batch) {
     __shared__ CtView sview[kFanViews];
-    __shared__ float red[NBT][kFanWarps][32];
+    __shared__ float red[PX * NBT][kFanWarps][32];
     const int lane = threadIdx.x, w = threadIdx.y, tid = w * 32 + lane;
-    const int i = (int)(blockIdx.x % tiles_x) * 8 + (lane & 7), j = (int)(blockIdx.x / tiles_x) * 4 + (lane >> 3);
+    const int i = (int)(blockIdx.x % tiles_x) * 8 + (lane & 7);
+    const int j = (int)(blockIdx.x / tiles_x) * (4 * PX) + (lane >> 3);
     const bool active = i < g.nx && j < g.ny;
     const size_t ystride = (size_t)g.nview * g.nu;
     for (int bt = blockIdx.y * NBT; bt < batch; bt += gridDim.y * NBT) {
         const TIn *ys = sino + bt * ystride;
-        float acc[NBT];
+        float acc[PX][NBT];
 #pragma unroll
-        for (int q = 0; q < NBT; ++q) acc[q] = 0.f;
+        for (int q = 0; q < PX * NBT; ++q) acc[q / NBT][q % NBT] = 0.f;
         for (int v0 = 0; v0 < g.nview; v0 += kFanViews) {
             const int n = min(kFanViews, g.nview - v0);
             __syncthreads();
@@ -211,17 +214,21 @@ fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sin
             __syncthreads();
             if (active)
                 for (int t = w; t < n; t += kFanWarps)
-                    fan_back_view<TIn, KIND, CURVED, RECON, NBT>(sview[t], g, ys + (size_t)(v0 + t) * g.nu,
-                                                                 ystride, i, j, acc);
+#pragma unroll
+                    for (int e = 0; e < PX; ++e)
+                        if (e == 0 || j + 4 * e < g.ny)
+                            fan_back_view<TIn, KIND, CURVED, RECON, NBT>(sview[t], g, ys + (size_t)(v0 + t) * g.nu,
+                                                                         ystride, i, j + 4 * e, acc[e]);
         }
 #pragma unroll
-        for (int q = 0; q < NBT; ++q) red[q][w][lane] = acc[q];
+        for (int q = 0; q < PX * NBT; ++q) red[q][w][lane] = acc[q / NBT][q % NBT];
         __syncthreads();
-        if (w < NBT && active) {
+        const int je = j + 4 * (w / NBT);
+        if (w < PX * NBT && active && je < g.ny) {
             float s = red[w][0][lane];
 #pragma unroll
             for (int q = 1; q < kFanWarps; ++q) s += red[w][q][lane];
-            st_out(g, vol, (size_t)(bt + w) * g.ny * g.nx + (size_t)j * g.nx + i, s, out_t);
+            st_out(g, vol, (size_t)(bt + w % NBT) * g.ny * g.nx + (size_t)je * g.nx + i, s, out_t);
         }
     }
 }
@@ -381,9 +388,15 @@ cudaError_t fan_fwd_k(const CtGrid &g, const CtView *views, const TIn *src, void
 template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
 cudaError_t fan_back_k(const CtGrid &g, const CtView *views, const TIn *src, void *out, int out_t, int batch,
                        cudaStream_t st) {
-    const int tiles_x = (g.nx + 7) / 8, tiles_y = (g.ny + 3) / 4;
+    // two pixels to a thread from 256 x 256 on (2048 warps of patches, before the
+    // split over views), where one image goes alone
+    const int px = NBT == 1 && (long long)g.nx * g.ny >= 65536 ? 2 : 1;
+    const int tiles_x = (g.nx + 7) / 8, tiles_y = (g.ny + 4 * px - 1) / (4 * px);
     dim3 blk(32, kFanWarps), grd((unsigned)tiles_x * (unsigned)tiles_y, (unsigned)std::min(batch / NBT, 65535));
-    fan_back<TIn, KIND, CURVED, RECON, NBT><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_x, batch);
+    if (px == 2)
+        fan_back<TIn, KIND, CURVED, RECON, NBT, NBT == 1 ? 2 : 1><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_x, batch);
+    else
+        fan_back<TIn, KIND, CURVED, RECON, NBT, 1><<<grd, blk, 0, st>>>(g, views, src, out, out_t, tiles_x, batch);
     return cudaGetLastError();
 }
 
