@@ -332,7 +332,9 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const int mn = min(af, al), mx = max(af, al) + NA - 1;
                 const int nmn = __shfl_down_sync(~0u, mn, 8), nmx = __shfl_down_sync(~0u, mx, 8);
                 const bool odd = __any_sync(~0u, hit && (lane & 7) && below == P.b0);
-                const bool near = __any_sync(~0u, lane < 24 && !(nmn > mx || mn > nmx));
+                // (two cells to spare: where a column hardly moves along u, its corners
+                // may do so in opposite directions, by less than a cell)
+                const bool near = __any_sync(~0u, lane < 24 && !(nmn > mx + 2 || mn > nmx + 2));
                 const int nph = (odd ? 2 : 1) * (near ? 4 : 1);
                 const int mine = (odd ? lane & 1 : 0) + (near ? (odd ? 2 : 1) * grp : 0);
                 const float val = P.amp * xv;
