@@ -54,11 +54,11 @@ FP32_LANES = 128  # FP32 FMA lanes per SM (Blackwell)
 # Counters of one `ncu --set full` capture of each kernel on this workload
 # (per launch): DRAM read + write bytes, L2 (lts__t_sectors x 32) bytes and the
 # L2 throughput peak implied by its percent-of-peak counter; src = sha256
-# prefix of the kernel's .cu at capture time (the bench reports null once the
+# prefix of the kernel's source at capture time (the bench reports null once the
 # source differs).
 NCU = {
-    "sf_fwd": {"dram_bytes": 935.3e6, "l2_bytes": 30.472e9, "l2_peak_gbs": 36275.0, "src": "27b5509270244406"},
-    "sf_back": {"dram_bytes": 353.1e6, "l2_bytes": 23.183e9, "l2_peak_gbs": 36275.0, "src": "27b5509270244406"},
+    "sf_fwd": {"dram_bytes": 1495.7e6, "l2_bytes": 28.577e9, "l2_peak_gbs": 36388.0, "src": "e6fc26b8654f6756"},
+    "sf_back": {"dram_bytes": 379.7e6, "l2_bytes": 11.380e9, "l2_peak_gbs": 36409.0, "src": "fd28c3c0410b5e93"},
 }
 
 
@@ -714,8 +714,8 @@ def main():
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     sm_mhz = (clk or {}).get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     fp32_peak = n_sm * FP32_LANES * 2 * sm_mhz * 1e6 / 1e12  # TFLOP/s at the sampled clock
-    dom, dom_ms, dom_src = ("sf_back", back_ms, "k_sf.cu") if back_ms >= fwd_ms else \
-        ("sf_fwd", fwd_ms, "k_sf.cu")
+    dom, dom_ms, dom_src = ("sf_back", back_ms, "k_circ_back.cuh") if back_ms >= fwd_ms else \
+        ("sf_fwd", fwd_ms, "k_circ_fwd.cuh")
     flops = SF_FLOPS_PER_UPDATE * spec.n_vox * spec.nview
     achieved = flops / (dom_ms * 1e-3) / 1e12
     nc = NCU.get(dom)
@@ -752,7 +752,7 @@ def main():
                          "frac": hbm_ach / hbm_peak, "bytes": "compulsory: read input once, write output once",
                          "peak_note": "of measured (MEASURED_PEAKS.json hbm_gbs)"},
         "e2e": e2e,
-        "gpu_launches": 3 * K,  # per step: z-major copy, SF forward, SF back
+        "gpu_launches": 3 * K,  # per step: volume copies, SF forward, SF back
         "clocks": clk,
     }
     if not args.no_serving:
