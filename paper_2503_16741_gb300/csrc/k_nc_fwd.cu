@@ -244,7 +244,7 @@ nc_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, 
 // but adds each weight once, where a gathering thread visits every voxel that
 // might reach its cells (five visits of 16 products per update for about eight
 // non-zero weights).  192^3 / 250 views / 384^2 FP16 SF-TR: gather 52.8 ms, tile
-// sums 27.1 ms (issue 77 % of slots, L1 79 %); 64^3 / 90 views DD 924 -> 405 us.
+// sums 27.2 ms (issue 77 % of slots, L1 79 %); 64^3 / 90 views DD 924 -> 415 us.
 template <int NA, int NB> struct ScTile {
     static constexpr int kMc = NA - 1, kMr = NB - 1;  // margins
     static constexpr int kPitch = (32 + 2 * kMc) | 1;
@@ -329,7 +329,8 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 // cell is monotone in k, and in l at a given k)
                 const int below = __shfl_up_sync(~0u, P.b0, 1, 8);
                 const int af = __shfl_sync(~0u, P.a0, 0, 8), al = __shfl_sync(~0u, P.a0, min(7, K1 - kc), 8);
-                const int mn = min(af, al), mx = max(af, al) + NA - 1;
+                const bool wide = __any_sync(~0u, hit && P.n > 4);
+                const int mn = min(af, al), mx = max(af, al) + (wide ? NA : min(NA, 4)) - 1;  // cells added to
                 const int nmn = __shfl_down_sync(~0u, mn, 8), nmx = __shfl_down_sync(~0u, mx, 8);
                 const bool odd = __any_sync(~0u, hit && (lane & 7) && below == P.b0);
                 // (two cells to spare: where a column hardly moves along u, its corners
@@ -340,13 +341,12 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const float val = P.amp * xv;
 #pragma unroll
                 for (int c = 0; c < NA; ++c) P.Fu[c] *= val;
-                const bool wide = __any_sync(~0u, hit && P.n > 4);
                 float *t0 = tile + (hit ? r0 * P_ + c0 : 0);
                 for (int ph = 0; ph < nph; ++ph) {
                     const bool go = hit && mine == ph;
 #pragma unroll
                     for (int q = 0; q < NB; ++q) {
-                        if (go) {
+                        if (go && P.Fv[q] != 0.f) {
 #pragma unroll
                             for (int c = 0; c < (NA < 4 ? NA : 4); ++c)
                                 t0[q * P_ + c] = fmaf(P.Fu[c], P.Fv[q], t0[q * P_ + c]);
