@@ -80,6 +80,17 @@ def test_circ_forward_matches_oracle(ct, det, size, proj):
     assert torch.equal(ct.forward(g.subset(views), x, proj), y[:, views])
 
 
+@pytest.mark.parametrize("views", [31, 32, 67, 150])  # 1, 2, 4 and 8 blocks share the views
+def test_sftt_back_with_shared_views_matches_oracle(ct, views):
+    spec = _spec("flat", 17, 9, 37, 33, 47, views, 3.4, 2.9)
+    g = ct.Geometry.from_spec(spec)
+    yd = torch.as_tensor(W.random_sino(spec, seed=2, batch=2) - 0.3, dtype=torch.float32).cuda()
+    x = ct.back(g, yd, "sftt")
+    for b in range(2):
+        _check(x[b].cpu().numpy(), oracle.back(spec, "sftt", yd[b].double().cpu().numpy()), "back")
+    assert torch.equal(x[1], ct.back(g, yd[1].contiguous(), "sftt"))
+
+
 @pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
 def test_a_bad_cell_stays_where_its_rays_go(ct, proj):
     """An infinite detector cell reaches only voxels whose footprint is near it."""
