@@ -104,9 +104,12 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
     if (KIND == FAN_VOX) {
         float fu, rden2;
         fan_point<CURVED>(V, cu, cn, fu, rden2);
+        // a pixel that projects beside the detector reads none of its cells (one of
+        // them may be infinite or NaN, which a weight of zero would not hide)
+        if (fu <= -1.f || fu >= (float)g.nu) return;
         const float af = floorf(fu), t = fu - af;
         const int a0 = (int)af;
-        // cells off the detector weigh zero and read a clamped address
+        // at its ends, the cell off the detector weighs zero and reads the one on it
         const float w0 = (unsigned)a0 < (unsigned)g.nu ? 1.f - t : 0.f;
         const float w1 = (unsigned)(a0 + 1) < (unsigned)g.nu ? t : 0.f;
         float amp = V.rc_w * rden2;

@@ -69,3 +69,24 @@ def test_fan_recon_back_matches_oracle(ct, det, proj):
     q = W.random_sino(spec, seed=3)[0]
     got = ct.back(g, torch.as_tensor(q[:, 0], dtype=torch.float32).cuda(), proj, mode="recon")
     _same(got.cpu().numpy(), oracle.back_recon(spec, q, proj).reshape(g.vol_shape), proj)
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("mode", ["proj", "recon"])
+@pytest.mark.parametrize("size", [(40, 33), (261, 259)], ids=["one-pixel", "two-pixels"])
+def test_a_bad_edge_cell_stays_on_the_detector(ct, det, mode, size):
+    """Voxel-driven back onto a detector that truncates the image: infinite cells at its ends reach only the pixels
+    that project beside them, not those whose rays pass beyond its end."""
+    spec = _spec(det, *size, 40, 12, size[0] * 1.6 / 40)
+    g = ct.Geometry.from_spec(spec)
+    y = torch.rand(g.sino_shape, device="cuda")
+    clean = ct.back(g, y, "voxel", mode=mode)
+    mask = np.zeros(spec.sino_shape)
+    for v, a in ((2, 0), (5, 39)):
+        y[v, a] = float("inf")
+        mask[v, 0, max(a - 1, 0):a + 2] = 1.0  # one cell of slack
+    bad = ct.back(g, y, "voxel", mode=mode)
+    ok = torch.isfinite(bad)
+    touched = oracle.back(spec, "voxel", mask).reshape(g.vol_shape) != 0
+    assert not ok.all() and torch.equal(bad[ok], clean[ok])
+    assert not (~ok.cpu().numpy() & ~touched).any()
