@@ -2,6 +2,8 @@
 (1 to 8 cells, and beyond), rows per voxel (below 1, 2, 4 and 8, and beyond),
 chunks, patches, tiles and columns with remainders, views split over a cluster
 and not, against the FP64 oracle at the FP32 path's bound."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -105,3 +107,58 @@ def test_a_bad_cell_stays_where_its_rays_go(ct, proj):
     mask = np.zeros(spec.sino_shape)
     mask[3, 38:43, 12:21] = 1.0
     assert not (~ok.cpu().numpy() & (oracle.back(spec, "sf", mask) == 0)).any()
+
+
+def _weighs(spec, proj, cells):
+    """Voxels with a weight on one of the cells (view, row, cell), positions on the detector uncertain by 1e-3 cell
+    (FP32 positions are good to 1e-4)."""
+    mask = np.zeros(spec.sino_shape)
+    for c in cells:
+        mask[c] = 1.0
+    out = np.zeros(spec.vol_shape, dtype=bool)
+    for su in (-1e-3, 0.0, 1e-3):
+        for sv in (-1e-3, 0.0, 1e-3):
+            moved = dataclasses.replace(spec, u_ofst=spec.u_ofst + su * spec.du, v_ofst=spec.v_ofst + sv * spec.dv)
+            out |= oracle.back(moved, proj, mask) != 0
+    return out
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("mode", ["proj", "recon"])
+@pytest.mark.parametrize("size", ["tall", "taller", "tallest"])
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+def test_a_bad_cell_reaches_the_voxels_it_weighs(ct, det, mode, size, proj):
+    """Voxels higher than a row read several rows; one that meets fewer of them is not reached by the others."""
+    spec = _spec(det, *SIZES[size])
+    g = ct.Geometry.from_spec(spec)
+    y = torch.rand(g.sino_shape, device="cuda")
+    clean = ct.back(g, y, proj, mode=mode)
+    nu, nv = spec.nu, spec.nv
+    cells = [(2, nv // 2, nu // 2), (3, nv // 2 + 5, 1), (4, nv // 2 - 5, nu - 2), (5, 1, nu // 2 + 3), (6, nv - 2, nu // 2)]
+    for c in cells:
+        y[c] = float("inf")
+    bad = ct.back(g, y, proj, mode=mode)
+    ok = torch.isfinite(bad)
+    assert not ok.all() and torch.equal(bad[ok], clean[ok])
+    assert not (~ok.cpu().numpy() & ~_weighs(spec, proj, cells)).any()
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("mode", ["proj", "recon"])
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+def test_a_bad_cell_near_the_detectors_end(ct, det, mode, proj):
+    """Windows moved onto a truncating detector do not read further than others: footprints of up to 8 cells by less
+    than a row take four cells (voxel-driven: its own two) and one row beyond their own."""
+    spec = _spec(det, 24, 24, 40, 40, 40, 9, 1.3, 3.1)
+    g = ct.Geometry.from_spec(spec)
+    y = torch.rand(g.sino_shape, device="cuda")
+    clean = ct.back(g, y, proj, mode=mode)
+    cells, near = [(2, 20, 1), (3, 18, 5), (4, 22, 34), (5, 21, 38)], []
+    for v, b, a in cells:
+        y[v, b, a] = float("inf")
+        w = 0 if proj == "voxel" else 3
+        near += [(v, r, c) for r in (b - 1, b, b + 1) for c in range(max(a - w, 0), min(a + w, 39) + 1)]
+    bad = ct.back(g, y, proj, mode=mode)
+    ok = torch.isfinite(bad)
+    assert not ok.all() and torch.equal(bad[ok], clean[ok])
+    assert not (~ok.cpu().numpy() & ~_weighs(spec, proj, near)).any()
