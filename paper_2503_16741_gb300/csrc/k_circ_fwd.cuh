@@ -115,8 +115,8 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
                 const float2 q = __ffma2_rn(wz, wz, make_float2(r2, r2));
                 v2 = __fmul2_rn(__fmul2_rn(q, make_float2(rsqrtf(q.x), rsqrtf(q.y))), v2);
             }
-            if constexpr (KIND == BK_VOX) {  // w to the row above, 1 - w to the row
-                const float2 up2 = __fmul2_rn(w2, v2), own2 = __ffma2_rn(up2, minus1, v2);
+            if constexpr (KIND == BK_VOX) {  // w to the row above, 1 - w to the row (v - w v would be NaN for an infinite v)
+                const float2 up2 = __fmul2_rn(w2, v2), own2 = __fmul2_rn(__ffma2_rn(w2, minus1, make_float2(1.f, 1.f)), v2);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int off = (int)(__float_as_uint(h ? m2.y : m2.x) << 10);

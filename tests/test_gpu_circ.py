@@ -162,3 +162,21 @@ def test_a_bad_cell_near_the_detectors_end(ct, det, mode, proj):
     ok = torch.isfinite(bad)
     assert not ok.all() and torch.equal(bad[ok], clean[ok])
     assert not (~ok.cpu().numpy() & ~_weighs(spec, proj, near)).any()
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("size", ["narrow-short", "tall"])
+def test_an_infinite_voxel_stays_infinite(ct, det, size):
+    """Voxel-driven forward: every cell that an infinite voxel weighs on is infinite, not NaN."""
+    spec = _spec(det, *SIZES[size])
+    g = ct.Geometry.from_spec(spec)
+    x = torch.rand(g.vol_shape, device="cuda")
+    clean = ct.forward(g, x, "voxel")
+    at = (spec.nz // 2, spec.ny // 2, spec.nx // 2)
+    x[at] = float("inf")
+    one = np.zeros(spec.vol_shape)
+    one[at] = 1.0
+    w = oracle.forward(spec, "voxel", one)
+    y = ct.forward(g, x, "voxel").cpu().numpy()
+    assert np.isposinf(y[w > 1e-3 * w.max()]).all()
+    assert np.array_equal(y[w == 0], clean.cpu().numpy()[w == 0])
