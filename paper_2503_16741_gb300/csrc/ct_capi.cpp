@@ -194,7 +194,6 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     g->du = d->du;
     g->dv = two_d ? 1.0 : d->dv;
     const bool curved = d->det == CT_DET_CURVED;
-    double min_v = 1e30;  // lower bound on a voxel's axial height (rows)
     g->host_views.resize(d->nview);
     const std::vector<double> dbeta = recon_dbetas(d, P);
 
@@ -288,10 +287,16 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
         V.m_sf_u = (float)bound(D / g->du, hx * std::fabs(eu.x) + hy * std::fabs(eu.y),
                                 hx * std::fabs(n.x) + hy * std::fabs(n.y), tu);
         V.m_sf_v = (float)bound(D / g->dv, hz * std::fabs(ev.z), hz * std::fabs(n.z), tv);
-        // the height 2 K |hz ev.z - t hz n.z| / (depth (1 - ..)) of the farthest voxel, seen at the widest ratio t,
-        // from its farthest transaxial corner
-        min_v = std::min(min_v, 0.999 * (2.0 * D / g->dv) * hz * (std::fabs(ev.z) - tv * std::fabs(n.z)) /
-                                    (bmax + hx * std::fabs(n.x) + hy * std::fabs(n.y)));
+        {
+            // Non-circular forward by tile sums:
+            // every axial footprint is more than half a row high, so that at most
+            // two voxels of a column start in a row: the height 2 K |hz ev.z - t hz n.z|
+            // / (depth (1 - ..)) of the farthest voxel, seen at the widest ratio t, from
+            // its farthest transaxial corner.
+            const double hdn = hx * std::fabs(n.x) + hy * std::fabs(n.y);
+            const double high = 0.999 * (2.0 * D / g->dv) * hz * (std::fabs(ev.z) - tv * std::fabs(n.z)) / (bmax + hdn);
+            V.nc_tile = high > 0.51 ? 1 : 0;
+        }
         // SF-TT: the z faces at the transaxial corners (a 2D row lies inside the
         // axial plateau, so its factor is 1 and the bound does not matter)
         V.m_tt_v = two_d ? 0.25f
@@ -321,12 +326,13 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     G.max_m_dd_u = 0.f;
     G.max_m_sf_v = 0.f;
     G.max_m_tt_v = 0.f;
-    G.min_v = (float)min_v;
+    G.nc_tile = G.nc_gather = 0;
     for (const CtView &V : g->host_views) {
         G.max_m_sf_u = std::max(G.max_m_sf_u, V.m_sf_u);
         G.max_m_dd_u = std::max(G.max_m_dd_u, V.m_dd_u);
         G.max_m_sf_v = std::max(G.max_m_sf_v, V.m_sf_v);
         G.max_m_tt_v = std::max(G.max_m_tt_v, V.m_tt_v);
+        (V.nc_tile ? G.nc_tile : G.nc_gather) = 1;
     }
 
     if (cudaGetDevice(&g->device) != cudaSuccess) {

@@ -39,7 +39,7 @@ struct alignas(16) CtView {
     // its height along e_v and n (mm; single precision, as the kernels use them)
     float cdu[4], cdn[4];
     float hzv, hzn;
-    float pad;
+    int nc_tile;      // the non-circular forward may sum the view by tiles (k_nc_fwd.cu)
 };
 static_assert(sizeof(CtView) == 52 * 4, "CtView layout");
 
@@ -57,7 +57,8 @@ struct CtGrid {
     float max_m_dd_u;  // largest per-view DD boundary bound (cells)
     float max_m_sf_v;  // largest per-view axial half-height bound (rows)
     float max_m_tt_v;  // largest per-view SF-TT axial bound (rows)
-    float min_v;       // lower bound on a voxel's axial height on the detector (rows)
+    int nc_tile;       // non-circular: some view has CtView::nc_tile set,
+    int nc_gather;     // some view has not
     float alpha, beta; // output epilogue: out = alpha * result + beta * out
 };
 

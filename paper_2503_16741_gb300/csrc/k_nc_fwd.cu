@@ -106,6 +106,7 @@ nc_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, 
     const int A0 = tu * 64, B0 = tv * 64;
     const int a = A0 + 4 * threadIdx.x, ty = threadIdx.y, rb = B0 + 4 * ty;
     const CtView &V = views[v];
+    if (V.nc_tile) return;  // the tile sums' (whole CTA)
     const int main_y = V.main_y;
     const SlabCoef sc = slab_coef(V, main_y);
     const float mu = (KIND == NC_DD ? V.m_dd_u : V.m_sf_u) + 0.5f + kSearchPad;
@@ -238,7 +239,11 @@ nc_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, 
 // footprint is at least a row high, so no two lanes of a column touch a cell in
 // the same step; where a height between half a row and one lets neighbours share
 // a row, or the four columns' cells are not apart, the lanes take turns (decided
-// by votes on the footprints themselves).  The order of every sum is fixed.
+// by votes on the footprints themselves).  The order of every sum is fixed, and
+// nothing that orders it depends on another view: which views are summed so is
+// decided view by view (CtView::nc_tile; the others take the gather above), and who
+// votes on sharing rows does not depend on the margins, which follow the scan's NA
+// and NB.
 //
 // Against the gather above it evaluates the same footprints (1.2 per update)
 // but adds each weight once, where a gathering thread visits every voxel that
@@ -254,7 +259,7 @@ constexpr int kScWarps = 4;
 
 template <typename TIn, int KIND, int NA, int NB>
 __global__ void __launch_bounds__(32 * kScWarps, 6)
-nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ volZ, void *__restrict__ sino,
+nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, bool zmajor, void *__restrict__ sino,
             int out_t, int tiles_u, int tiles_v, int R) {
     using Tile = ScTile<NA, NB>;
     constexpr int P_ = Tile::kPitch;
@@ -286,14 +291,17 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
     }
     for (int q = lane; q < Tile::floats(R); q += 32) tile[q] = 0.f;
     __syncthreads();
+    if (!V.nc_tile) return;  // the gather's (whole CTA)
     const int main_y = V.main_y;
     const SlabCoef sc = slab_coef(V, main_y);
     const int nslab = main_y ? g.ny : g.nx, nlat = main_y ? g.nx : g.ny;
     const float hl = main_y ? g.dx : g.dy, hs = main_y ? g.dy : g.dx;
     const float ol = main_y ? V.o[0] : V.o[1], os = main_y ? V.o[1] : V.o[0];
-    // strides of the copy along the lateral axis and the slabs
-    const size_t pl = (size_t)g.nz * (main_y ? 1 : g.nx), ps = (size_t)g.nz * (main_y ? g.nx : 1);
-    const TIn *xz = volZ + (size_t)bt * g.nx * g.ny * g.nz;
+    // strides along z, the lateral axis and the slabs: of the z-major copy, or of the
+    // volume itself where the copy could not be had
+    const size_t pk = zmajor ? 1 : (size_t)g.nx * g.ny, pc = zmajor ? g.nz : 1;
+    const size_t pl = pc * (main_y ? 1 : g.nx), ps = pc * (main_y ? g.nx : 1);
+    const TIn *xz = vol + (size_t)bt * g.nx * g.ny * g.nz;
     const int grp = lane >> 3;
     for (int s = w; s < nslab; s += kScWarps) {
         int L0, L1, K0, K1;
@@ -305,7 +313,7 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
         for (int kc = K0; kc <= K1; kc += 8) {
             const int k = kc + (lane & 7);
             const float fk = (float)k;
-            const TIn *xk = xz + s * ps + l0 * pl + k;
+            const TIn *xk = xz + s * ps + l0 * pl + k * pk;
             for (int t = 0; t < nq; ++t, xk += pl) {
                 const bool in = k <= K1 && l0 + t <= L1;
                 const float xv = in ? ld(xk, 0) : 0.f;
@@ -332,7 +340,7 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const bool wide = __any_sync(~0u, hit && P.n > 4);
                 const int mn = min(af, al), mx = max(af, al) + (wide ? NA : min(NA, 4)) - 1;  // cells added to
                 const int nmn = __shfl_down_sync(~0u, mn, 8), nmx = __shfl_down_sync(~0u, mx, 8);
-                const bool odd = __any_sync(~0u, hit && (lane & 7) && below == P.b0);
+                const bool odd = __any_sync(~0u, in && (lane & 7) && below == P.b0);
                 // (two cells to spare: where a column hardly moves along u, its corners
                 // may do so in opposite directions, by less than a cell)
                 const bool near = __any_sync(~0u, lane < 24 && !(nmn > mx + 2 || mn > nmx + 2));
@@ -388,10 +396,7 @@ template <typename TIn, int KIND, int NA, int NB> struct NcFwd {
     static cudaError_t go(const CtGrid &g, const CtView *views, const void *in, void *out, int out_t, int batch,
                           cudaStream_t st) {
         const TIn *src = static_cast<const TIn *>(in);
-        const size_t smem = sizeof(NcCache<NA>);
-        cudaError_t e = cudaFuncSetAttribute(nc_fwd<TIn, KIND, NA, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
+        cudaError_t e = cudaSuccess;
         // a z-major copy of the volume (pooled workspace) makes each round's
         // reads contiguous along k; without it the reads are strided
         TIn *xZ = nullptr;
@@ -404,32 +409,30 @@ template <typename TIn, int KIND, int NA, int NB> struct NcFwd {
             return e;
         }
         const size_t nvb = (g.nview + kNcViewBlock - 1) / kNcViewBlock;
-        // tile sums where every axial footprint is more than half a row high
-        // (so that at most two voxels of a column start in a row) and the copy
-        // could be had; the gather otherwise
-        if (xZ && g.min_v > 0.51f) {
+        if (g.nc_tile) {  // the views that allow tile sums
             const int R = sc_rows(g);
             const int tiles_c = (g.nu + 31) / 32, tiles_r = (g.nv + R - 1) / R;
             const size_t sm = sizeof(float) * kScWarps * (size_t)ScTile<NA, NB>::floats(R);
             e = cudaFuncSetAttribute(nc_fwd_tile<TIn, KIND, NA, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
             if (e == cudaSuccess) {
                 const dim3 grd((unsigned)((size_t)kNcViewBlock * tiles_c * tiles_r * nvb * batch));
-                nc_fwd_tile<TIn, KIND, NA, NB><<<grd, dim3(32, kScWarps), sm, st>>>(g, views, xZ, out, out_t, tiles_c,
-                                                                                   tiles_r, R);
+                nc_fwd_tile<TIn, KIND, NA, NB><<<grd, dim3(32, kScWarps), sm, st>>>(g, views, xZ ? xZ : src, xZ != nullptr, out,
+                                                                                   out_t, tiles_c, tiles_r, R);
                 e = cudaGetLastError();
             }
-            const cudaError_t ef = workspace_free(xZ, st);
-            return e != cudaSuccess ? e : ef;
         }
-        const int tiles_u = (g.nu + 63) / 64, tiles_v = (g.nv + 63) / 64;
-        dim3 blk(16, 16), grd((unsigned)((size_t)kNcViewBlock * tiles_u * tiles_v * nvb * batch));
-        nc_fwd<TIn, KIND, NA, NB><<<grd, blk, smem, st>>>(g, views, src, xZ, out, out_t, tiles_u, tiles_v);
-        e = cudaGetLastError();
-        if (xZ) {
-            const cudaError_t ef = workspace_free(xZ, st);
-            if (e == cudaSuccess) e = ef;
+        if (e == cudaSuccess && g.nc_gather) {  // the others
+            const size_t smem = sizeof(NcCache<NA>);
+            e = cudaFuncSetAttribute(nc_fwd<TIn, KIND, NA, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e == cudaSuccess) {
+                const int tiles_u = (g.nu + 63) / 64, tiles_v = (g.nv + 63) / 64;
+                dim3 blk(16, 16), grd((unsigned)((size_t)kNcViewBlock * tiles_u * tiles_v * nvb * batch));
+                nc_fwd<TIn, KIND, NA, NB><<<grd, blk, smem, st>>>(g, views, src, xZ, out, out_t, tiles_u, tiles_v);
+                e = cudaGetLastError();
+            }
         }
-        return e;
+        const cudaError_t ef = workspace_free(xZ, st);
+        return e != cudaSuccess ? e : ef;
     }
 };
 }  // namespace

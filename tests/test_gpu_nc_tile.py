@@ -44,3 +44,33 @@ def test_noncircular_forward_matches_oracle(size, proj):
     assert torch.equal(y[1], ct.forward(g, x[1].contiguous(), proj))
     views = [0, 3, 34]
     assert torch.equal(ct.forward(g.subset(views), x, proj), y[:, views])
+
+
+# du, dv: half of the views at magnification 2, half at 1.33
+MIXED = {
+    "kernels": (2.9, 3.6),  # axial footprints of about 0.7 and 0.48 rows: tile sums and the gather
+    "cells": (1.6, 2.0),    # 6 and 4 cells
+    "rows": (1.6, 1.25),    # 4 and 3 rows
+}
+
+
+@pytest.mark.parametrize("proj", ["sf", "dd", "sftt"])
+@pytest.mark.parametrize("mix", MIXED)
+def test_a_view_does_not_depend_on_the_others(mix, proj):
+    """Views on either side of a dispatch rule: each has the same projection alone, among its like and in the mix."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_16741_gb300 as ct
+    du, dv = MIXED[mix]
+    nview = 38
+    th = 0.1 + 2 * np.pi * np.arange(nview) / nview
+    sad = np.where(np.arange(nview) % 2 == 0, 320.0, 480.0)
+    spec = W.GeometrySpec("noncirc3d", "flat", 37, 33, 29, 1.6, 1.6, 1.3, 75, 50, du, dv, nview, theta=th,
+                          phi=0.05 * np.cos(2 * th), psi=0.02 * np.sin(3 * th), sad=sad, sdd=640.0, x_src=1.2,
+                          z_src=-2.0, u_ofst=-2.6, v_ofst=1.7, x_ofst=2.0, y_ofst=-1.0, z_ofst=1.5)
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=3)[0] - 0.3, dtype=torch.float32).cuda()
+    y = ct.forward(g, x, proj)
+    assert rel_l2(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy())) <= TOL_F32
+    for views in (list(range(0, nview, 2)), list(range(1, nview, 2)), [4], [5]):
+        assert torch.equal(ct.forward(g.subset(views), x, proj), y[views])
