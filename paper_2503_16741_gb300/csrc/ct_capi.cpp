@@ -288,14 +288,20 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
                                 hx * std::fabs(n.x) + hy * std::fabs(n.y), tu);
         V.m_sf_v = (float)bound(D / g->dv, hz * std::fabs(ev.z), hz * std::fabs(n.z), tv);
         {
-            // Non-circular forward by tile sums:
-            // every axial footprint is more than half a row high, so that at most
+            // Non-circular forward by tile sums: two conditions on the view.
+            // (1) Every axial footprint is more than half a row high, so that at most
             // two voxels of a column start in a row: the height 2 K |hz ev.z - t hz n.z|
             // / (depth (1 - ..)) of the farthest voxel, seen at the widest ratio t, from
             // its farthest transaxial corner.
-            const double hdn = hx * std::fabs(n.x) + hy * std::fabs(n.y);
+            const double hdu = hx * std::fabs(eu.x) + hy * std::fabs(eu.y), hdn = hx * std::fabs(n.x) + hy * std::fabs(n.y);
             const double high = 0.999 * (2.0 * D / g->dv) * hz * (std::fabs(ev.z) - tv * std::fabs(n.z)) / (bmax + hdn);
-            V.nc_tile = high > 0.51 ? 1 : 0;
+            // (2) Over eight voxels of a column the corners' offsets from the centre,
+            // p = K (du - r dn) / (depth + dn) with r the centre's ratio, change by less
+            // than a cell: with U, N the steps of w.e_u and w.n from voxel to voxel,
+            // |dr| <= 7 (U + t N) / depth and |d depth| <= 7 N.
+            const double U = 2 * hz * std::fabs(eu.z), N = 2 * hz * std::fabs(n.z);
+            const double shift = 7 * (D / g->du) * ((U + tu * N) * hdn + (hdu + tu * hdn) * N) / (bmin * bmin);
+            V.nc_tile = high > 0.51 && shift < 0.9 ? 1 : 0;
         }
         // SF-TT: the z faces at the transaxial corners (a 2D row lies inside the
         // axial plateau, so its factor is 1 and the bound does not matter)

@@ -245,6 +245,16 @@ nc_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, 
 // votes on sharing rows does not depend on the margins, which follow the scan's NA
 // and NB.
 //
+// Why two lanes never add to one cell in the same step.  The cells a column adds
+// to over its eight voxels lie between a0 and a0 + 3 (NA - 1) of its footprints.
+// Each transaxial corner moves one way along u with k, so the lowest a0 is that of
+// the first or the last voxel, up to one cell of rounding.  The highest may exceed
+// both, where corners move opposite ways, by no more than the corners' offsets from
+// the centre change, since the centre itself moves one way: less than a cell by the
+// host's condition on nc_tile.  So ranges taken from the end voxels that are more
+// than two cells apart do not meet; and as centres are monotone along the slab,
+// neighbouring groups that are apart leave all four apart.
+//
 // Against the gather above it evaluates the same footprints (1.2 per update)
 // but adds each weight once, where a gathering thread visits every voxel that
 // might reach its cells (five visits of 16 products per update for about eight
@@ -341,8 +351,6 @@ nc_fwd_tile(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
                 const int mn = min(af, al), mx = max(af, al) + (wide ? NA : min(NA, 4)) - 1;  // cells added to
                 const int nmn = __shfl_down_sync(~0u, mn, 8), nmx = __shfl_down_sync(~0u, mx, 8);
                 const bool odd = __any_sync(~0u, in && (lane & 7) && below == P.b0);
-                // (two cells to spare: where a column hardly moves along u, its corners
-                // may do so in opposite directions, by less than a cell)
                 const bool near = __any_sync(~0u, lane < 24 && !(nmn > mx + 2 || mn > nmx + 2));
                 const int nph = (odd ? 2 : 1) * (near ? 4 : 1);
                 const int mine = (odd ? lane & 1 : 0) + (near ? (odd ? 2 : 1) * grp : 0);

@@ -74,3 +74,22 @@ def test_a_view_does_not_depend_on_the_others(mix, proj):
     assert rel_l2(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy())) <= TOL_F32
     for views in (list(range(0, nview, 2)), list(range(1, nview, 2)), [4], [5]):
         assert torch.equal(ct.forward(g.subset(views), x, proj), y[views])
+
+
+@pytest.mark.parametrize("proj", ["sf", "dd"])
+def test_steep_views_near_the_source(proj):
+    """Views whose footprints change by more than a cell along a column (a small volume close to the source, the
+    detector rolled by 51 degrees) beside upright ones: either forward, in one scan."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2503_16741_gb300 as ct
+    th = np.array([0.37, 1.2, 2.9, 4.4])
+    spec = W.GeometrySpec("noncirc3d", "flat", 8, 8, 6, 1.6, 1.6, 1.96, 50, 44, 2.4, 2.5, 4, theta=th,
+                          phi=np.array([0.115, 0.0, 0.115, 0.05]), psi=np.array([0.892, 0.0, 0.892, 0.02]),
+                          sad=np.array([20.4, 30.0, 20.4, 30.0]), sdd=60.8)
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=5)[0] - 0.3, dtype=torch.float32).cuda()
+    y = ct.forward(g, x, proj)
+    assert rel_l2(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy())) <= TOL_F32
+    for views in ([0, 2], [1, 3], [2]):
+        assert torch.equal(ct.forward(g.subset(views), x, proj), y[views])
