@@ -2,7 +2,7 @@
 // projectors whose weight is transaxial x axial: SF-TR, DD and voxel-driven
 // (Sec. 2.3; Long, Fessler & Balter 2010; De Man & Basu 2004; Peters 1981).
 //
-// CTA = 64 or 32 cells x BV = 64 or 32 rows of one view, 256 threads.  Work
+// CTA = 8 to 64 cells x BV = 64, 32 or 8 rows of one view, 256 threads.  Work
 // items are the voxel columns (slab s, lateral l) whose footprint can reach the
 // tile, taken 256 at a time.
 //   stage 1: thread = item; it forms the column's transaxial weights (NT
@@ -42,6 +42,17 @@
 
 namespace ctp {
 
+// CTAs of tiles `cells` wide and 64 rows high, and a wave of them (three to an SM)
+inline long long circ_fwd_ctas(const CtGrid &g, int cells, int batch) {
+    return (long long)((g.nu + cells - 1) / cells) * ((g.nv + 63) / 64) * g.nview * batch;
+}
+constexpr long long kFwdWave = 3 * 152;
+// Volumes of at most 32^3 voxels in calls of few CTAs are read in place: the copies
+// would cost such a call an allocation and a launch, a third of its time.
+inline bool circ_fwd_direct(const CtGrid &g, int batch) {
+    return (long long)g.nx * g.ny * g.nz * batch <= 32768 && circ_fwd_ctas(g, 32, batch) < kFwdWave;
+}
+
 namespace {
 constexpr int kFwdItems = 256;  // items of a round = threads
 constexpr int kFwdSeg = 256;    // slabs of a segment
@@ -58,6 +69,19 @@ template <int BV, int NT> struct CircFwdSmem {
 };
 }  // namespace
 
+// Voxels k .. k + 3 of a column from the address of voxel k: four in a row in a
+// copy, which is padded with zeros, or (DIRECT) a slice apart in the volume itself.
+template <bool DIRECT, typename TIn>
+__device__ __forceinline__ void walk_load(const CtGrid &g, const TIn *__restrict__ p, int k, float (&x)[4]) {
+    if constexpr (DIRECT) {
+        const size_t zs = (size_t)g.nx * g.ny;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) x[t] = k + t < g.nz ? ld(p, t * zs) : 0.f;
+    } else {
+        ld4(p, x);
+    }
+}
+
 // Stage 1's walk.  Voxel k's rectangle covers rows [p, p + sv] with p = lo +
 // (k - ks) sv (rows from the tile's row 0; VOX: p is its centre's row minus one
 // half), and consecutive rectangles abut, so every row's sum is complete when
@@ -65,7 +89,7 @@ template <int BV, int NT> struct CircFwdSmem {
 // does is read off the rounded edge that the next voxel starts from, so the
 // two agree whatever the rounding.)  TALL: a voxel may cover whole rows.
 // Voxels outside [k0, k1] reach no row of the tile.
-template <typename TIn, int KIND, int BV, bool TALL>
+template <typename TIn, int KIND, int BV, bool TALL, bool DIRECT>
 __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict__ cz, size_t pitch, float (&xa)[4],
                                           int k0, int k1, float sv, float fv0, float r2, float oz, int B0,
                                           float (&Z)[BV][kFwdItems], int tid) {
@@ -164,12 +188,12 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
     const TIn *cq = cz + (size_t)(ks >> 2) * pitch;
     float xb[4];
     float kk = 0.f;
-    for (int left = k1 - ks;; left -= 8, kk += 8.f) {
-        if (left >= 4) ld4(cq + pitch, xb);
+    for (int left = k1 - ks, k = ks + 4;; left -= 8, k += 8, kk += 8.f) {
+        if (left >= 4) walk_load<DIRECT>(g, cq + pitch, k, xb);
         quad(kk, xa);
         if (left < 4) break;
         cq += 2 * pitch;
-        if (left >= 8) ld4(cq, xa);
+        if (left >= 8) walk_load<DIRECT>(g, cq, k + 4, xa);
         quad(kk + 4.f, xb);
         if (left < 8) break;
     }
@@ -182,11 +206,12 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
     for (int q = max(r, 0); q < BV; ++q) Z[q][tid] = 0.f;
 }
 
-// CTA = CELLS cells x BV rows, CELLS / 32 x NG warps, RPT rows to a thread.
+// CTA = CELLS cells x BV rows, RPT rows to a thread, NG threads to a cell.
 // (BV = 64: 3 blocks per SM by shared memory and 80 registers; 32 x 32: 4 at 64)
-template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL>
-__global__ void __launch_bounds__(256, BV == 32 ? 4 : 3)
-circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ volZ, int nzp, void *__restrict__ sino,
+// DIRECT: the volume itself instead of its copies.
+template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL, bool DIRECT>
+__global__ void __launch_bounds__(256, BV == 64 ? 3 : 4)
+circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, int nzp, void *__restrict__ sino,
          int out_t, int tiles_u, int tiles_v) {
     constexpr int NG = 256 / CELLS, RPT = BV / NG;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -198,8 +223,8 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
     const int bt = bx / g.nview;
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const int A0 = tu * CELLS, B0 = tv * BV, Bn = min(BV, g.nv - B0);  // rows of the tile on the detector
-    const int ac = (int)(threadIdx.y % (CELLS / 32)) * 32 + (int)threadIdx.x;  // the thread's cell in the tile
-    const int rg = (int)threadIdx.y / (CELLS / 32);                          // and its rows rg, rg + NG, ..
+    // the thread's cell in the tile, and its rows rg, rg + NG, ..
+    const int ac = CELLS == 32 ? (int)threadIdx.x : tid % CELLS, rg = CELLS == 32 ? (int)threadIdx.y : tid / CELLS;
     const int a = A0 + ac;
     const CtView &V = views[v];
     const int main_y = V.main_y;
@@ -209,7 +234,7 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
     const float mv = KIND == BK_VOX ? 1.f + kSearchPad : V.m_sf_v + 0.5f + kSearchPad;
     const int nslab = main_y ? g.ny : g.nx, nlat = main_y ? g.nx : g.ny;
     // the copy whose columns are adjacent along the view's lateral axis
-    const TIn *xz = volZ + ((size_t)bt * 2 + (main_y ? 0 : 1)) * g.nx * g.ny * nzp;
+    const TIn *xz = vol + (DIRECT ? (size_t)bt * g.nz : ((size_t)bt * 2 + (main_y ? 0 : 1)) * nzp) * g.nx * g.ny;
     // the two lines of constant u that bound the cell's reach: lateral index = p + s slab
     float p1, s1, p2, s2;
     {
@@ -285,10 +310,10 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                 const float rsv = __fdividef(1.f, sv);
                 const int k0 = max(0, (int)ceilf(((float)B0 - fv0 - hw) * rsv - 1e-3f));
                 const int k1 = min(g.nz - 1, (int)floorf(((float)(B0 + Bn - 1) - fv0 + hw) * rsv + 1e-3f));
-                const TIn *cz = xz + 4 * ((size_t)s * nlat + l);
+                const TIn *cz = xz + (DIRECT ? (size_t)j * g.nx + i : 4 * ((size_t)s * nlat + l));
                 const size_t pitch = 4 * (size_t)g.nx * g.ny;
                 float x4[4] = {0.f, 0.f, 0.f, 0.f};  // on its way while the weights are formed
-                if (k0 <= k1) ld4(cz + (size_t)(k0 >> 2) * pitch, x4);
+                if (k0 <= k1) walk_load<DIRECT>(g, cz + (size_t)(k0 >> 2) * pitch, k0 & ~3, x4);
                 if constexpr (KIND == BK_VOX) {
                     const float fu = CURVED ? fmaf(V.Ku, atan2f(cu, cn), V.Cu) : fmaf(V.Ku, cu * rden, V.Cu);
                     const float af = floorf(fu), amp = vx_amp(g, V, 1.f, CURVED ? den2 * rden : cn);
@@ -316,8 +341,8 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
                     S.a0[tid] = (short)(aref + d0 - A0);
                 }
                 if (k0 <= k1)
-                    circ_walk<TIn, KIND, BV, TALL>(g, cz, pitch, x4, k0, k1, sv, fv0, fmaf(wx, wx, wy * wy), V.o[2], B0,
-                                                   S.Z, tid);
+                    circ_walk<TIn, KIND, BV, TALL, DIRECT>(g, cz, pitch, x4, k0, k1, sv, fv0, fmaf(wx, wx, wy * wy),
+                                                           V.o[2], B0, S.Z, tid);
                 else
                     for (int r = 0; r < BV; ++r) S.Z[r][tid] = 0.f;
             }
@@ -371,33 +396,54 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
 
 // ------------------------------------------------------------ launchers
 namespace {
-template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL>
-cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
+template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL, bool DIRECT = false>
+cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *x, int nzp, void *out, int out_t, int batch,
                         cudaStream_t st) {
     const int tiles_u = (g.nu + CELLS - 1) / CELLS, tiles_v = (g.nv + BV - 1) / BV;
     const size_t smem = sizeof(CircFwdSmem<BV, NT>);
-    auto kern = circ_fwd<TIn, KIND, CURVED, CELLS, BV, NT, TALL>;
+    auto kern = circ_fwd<TIn, KIND, CURVED, CELLS, BV, NT, TALL, DIRECT>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((unsigned)((size_t)tiles_u * tiles_v * g.nview * batch)), dim3(32, 8), smem, st>>>(
-        g, views, xZ, nzp, out, out_t, tiles_u, tiles_v);
+        g, views, x, nzp, out, out_t, tiles_u, tiles_v);
     return cudaGetLastError();
 }
 
-// Tiles of 64 cells x 64 rows, where a thread of stage 2 sums 16 rows and so
-// shares what it does per column among twice the rows of a 32 x 64 tile (256^3 /
-// 360 views SF-TR 11.4 -> 10.7 ms, 161^2 x 155 / 607 views 5.6 -> 5.1 ms); 32 x 64
-// where voxels may cover whole rows, whose walk takes the registers (64 x 64
-// spills: 183^2 x 157 / 231 views DD 3.7 -> 4.2 ms); 32 x 32 for a short detector
-// and for one of few tiles (more CTAs of a small scan).  The choice does not
-// depend on the views or the batch, so a view's result does not either.
+// The tile.  Its height follows the detector alone, since a column's walk starts
+// where the tile does: 64 rows, or fewer where they hold the detector (which leaves
+// the walk as it is).  64 even for a detector that is cut into few tiles: a column's
+// set-up is shared by twice the rows of a 32-row tile (64^3 / 360 views / 128 x 96
+// SF-TR 452 -> 353 us, curved 256^2 x 64 / 246 views / 444 x 64 DD 3813 -> 3040 us);
+// 8 for a short one (96^2 x 8 / 143 views / 150 x 4 SF-TR 178 -> 127 us against 32).
+// Its width decides how many CTAs there are and changes no bit of a result, so it
+// may follow the views and the batch.  64 cells are the fastest where they fill the
+// chip: a thread of stage 2 sums 16 rows and shares what it does per column among
+// them (256^3 / 360 views SF-TR 11.4 -> 10.5 ms against 32).  But a CTA takes the time
+// of its columns in all slabs, however few others run: below two waves (three CTAs to
+// an SM) 32 cells, below one 16, below a quarter 8.  256^3 / 512 x 384 SF-TR, 64, 32
+// and 16 cells: 1 view 1147, 509, 320 us; 8 views 1143, 653, 574; 16 views 1138, 829,
+// 859; 32 views 1462, 1304, 1441; 64 views 2360, 2312, 2687.  64^3 / 1 view / 128 x 96
+// DD, 16 and 8 cells: 59, 49 us.  (16 rows by 16 cells in their place: better for one
+// view, up to twice the time for a few.)  Voxels that may cover whole rows have a walk
+// that spills at 64 x 64 (183^2 x 157 / 231 views DD 3.7 -> 4.2 ms).
 template <typename TIn, int KIND, bool CURVED, int NT, bool TALL>
 cudaError_t circ_fwd_rpt(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
                          cudaStream_t st) {
-    const int tiles = ((g.nu + 31) / 32) * ((g.nv + 63) / 64);
-    if (g.nv > 32 && tiles > 16)
-        return circ_fwd_go<TIn, KIND, CURVED, TALL ? 32 : 64, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
-    return circ_fwd_go<TIn, KIND, CURVED, 32, 32, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+    // (TALL everywhere: one kernel serves either height of voxels in small calls)
+    const bool direct = circ_fwd_direct(g, batch);
+    if (g.nv <= 8)
+        return direct ? circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true, true>(g, views, xZ, nzp, out, out_t, batch, st)
+                      : circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true>(g, views, xZ, nzp, out, out_t, batch, st);
+    if (direct) return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, true, true>(g, views, xZ, nzp, out, out_t, batch, st);
+    if (circ_fwd_ctas(g, 16, batch) < kFwdWave / 2)
+        return circ_fwd_go<TIn, KIND, CURVED, 8, 64, NT, true>(g, views, xZ, nzp, out, out_t, batch, st);
+    if (circ_fwd_ctas(g, 32, batch) < kFwdWave)
+        return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+    if (g.nv <= 32) return circ_fwd_go<TIn, KIND, CURVED, 32, 32, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+    if constexpr (!TALL)
+        if (circ_fwd_ctas(g, 64, batch) >= 2 * kFwdWave)
+            return circ_fwd_go<TIn, KIND, CURVED, 64, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+    return circ_fwd_go<TIn, KIND, CURVED, 32, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
 }
 
 template <typename TIn, int KIND, bool CURVED, int NT>

@@ -50,12 +50,21 @@ bool circ_fwd_fits(const CtGrid &g, int kind, int batch) {
 }
 
 size_t circ_fwd_workspace(const CtGrid &g, int batch, int elem_bytes) {
+    if (circ_fwd_direct(g, batch)) return 0;
     return (size_t)2 * g.nx * g.ny * zmajor_pitch(g) * batch * elem_bytes;
 }
 
 cudaError_t launch_circ_fwd(int kind, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                             void *out, int batch, cudaStream_t st) {
     const int nzp = zmajor_pitch(g), isz = in_t == 0 ? 4 : 2;
+    auto go = [&](const void *x) {
+        switch (in_t) {
+        case 0: return circ_fwd_f32(kind, g, views, x, nzp, out, out_t, batch, st);
+        case 1: return circ_fwd_f16(kind, g, views, x, nzp, out, out_t, batch, st);
+        default: return circ_fwd_bf16(kind, g, views, x, nzp, out, out_t, batch, st);
+        }
+    };
+    if (circ_fwd_direct(g, batch)) return go(in);
     void *xZ = nullptr;
     cudaError_t e = workspace_alloc(&xZ, circ_fwd_workspace(g, batch, isz), st);
     if (e != cudaSuccess) return e;
@@ -67,13 +76,7 @@ cudaError_t launch_circ_fwd(int kind, const CtGrid &g, const CtView *views, int 
         quad_copies<__half><<<tg, dim3(32, 8), 0, st>>>(static_cast<const __half *>(in), static_cast<__half *>(xZ),
                                                         g.nx, g.ny, g.nz, nzp);
     e = cudaGetLastError();
-    if (e == cudaSuccess) {
-        switch (in_t) {
-        case 0: e = circ_fwd_f32(kind, g, views, xZ, nzp, out, out_t, batch, st); break;
-        case 1: e = circ_fwd_f16(kind, g, views, xZ, nzp, out, out_t, batch, st); break;
-        default: e = circ_fwd_bf16(kind, g, views, xZ, nzp, out, out_t, batch, st); break;
-        }
-    }
+    if (e == cudaSuccess) e = go(xZ);
     const cudaError_t ef = workspace_free(xZ, st);
     return e != cudaSuccess ? e : ef;
 }

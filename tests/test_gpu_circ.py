@@ -180,3 +180,47 @@ def test_an_infinite_voxel_stays_infinite(ct, det, size):
     y = ct.forward(g, x, "voxel").cpu().numpy()
     assert np.isposinf(y[w > 1e-3 * w.max()]).all()
     assert np.array_equal(y[w == 0], clean.cpu().numpy()[w == 0])
+
+
+# nx, ny, nz, nu, nv, views, du, dv, half voxel heights above and below half a row
+WIDTHS = {
+    "short": (33, 17, 9, 150, 7, 130, 1.0, 3.2),     # one tile of 8 rows
+    "one-tile": (33, 17, 24, 150, 30, 130, 1.0, 3.2),  # one tile of 32 rows (64 when few)
+    "large": (41, 23, 170, 150, 150, 104, 1.0, 3.2),   # tiles of 64 cells, 64 + 64 + 22 rows
+    "tall": (41, 23, 60, 150, 150, 60, 1.0, 1.3),      # voxels of 1.9 to 2.2 rows
+}
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("size", WIDTHS)
+@pytest.mark.parametrize("proj,dtype", [("sf", torch.float32), ("dd", torch.float32), ("voxel", torch.float32),
+                                        ("sf", torch.float16)], ids=["sf", "dd", "voxel", "sf-f16"])
+def test_circ_forward_at_every_tile_width(ct, det, size, proj, dtype):
+    """The width of a tile follows the number of views and changes nothing: all views, some and one agree bit for bit,
+    and with the oracle."""
+    spec = _spec(det, *WIDTHS[size])
+    half = [0.5 * spec.dz * 640.0 / spec.dv / r for r in (320.0 + 45.0, 320.0 - 45.0)]  # in rows, farthest and nearest
+    assert (half[1] < 0.5) == (size != "tall") and (size != "tall" or half[0] > 0.5)
+    tiles = -(-spec.nu // 64) * -(-spec.nv // 64) * spec.nview
+    assert size != "large" or tiles >= 2 * 3 * 152  # tiles of 64 cells
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=2)[0] - 0.3, dtype=torch.float32).cuda().to(dtype)
+    y = ct.forward(g, x, proj, out_dtype=torch.float32)
+    _check(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy()), "forward")
+    for views in (list(range(0, spec.nview, 3)), [1], [spec.nview - 1]):
+        assert torch.equal(ct.forward(g.subset(views), x, proj, out_dtype=torch.float32), y[views])
+
+
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel"])
+@pytest.mark.parametrize("du,dv", [(2.6, 3.2), (1.5, 1.5)])
+def test_a_view_does_not_depend_on_the_others(ct, proj, du, dv):
+    """Views at two magnifications: voxels below and above a row, footprints of different widths."""
+    nview = 20
+    sad = np.where(np.arange(nview) % 2 == 0, 320.0, 200.0)
+    spec = dataclasses.replace(_spec("flat", 25, 19, 41, 70, 75, nview, du, dv), sad=sad)
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=4)[0] - 0.3, dtype=torch.float32).cuda()
+    y = ct.forward(g, x, proj)
+    _check(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy()), "forward")
+    for views in (list(range(0, nview, 2)), list(range(1, nview, 2)), [4]):
+        assert torch.equal(ct.forward(g.subset(views), x, proj), y[views])
