@@ -107,7 +107,8 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
     const float wz0 = fmaf((float)ks, g.dz, oz);
     // rows below the walk's first one
     int open = (int)(__float_as_uint(lo + 12582912.f) << 10);  // byte offset of the open row
-    for (int q = 0; q < min(open >> 10, BV); ++q) Z[q][tid] = 0.f;
+    // (VOX: rows between two voxels' rows, which the walk passes over)
+    for (int q = 0; q < (TALL && KIND == BK_VOX && sv > 1.9f ? BV : min(open >> 10, BV)); ++q) Z[q][tid] = 0.f;
     float acc = 0.f, acc1 = 0.f;  // sum of the open row (VOX: and of the next)
     const unsigned zt = (unsigned)__cvta_generic_to_shared(&Z[0][tid]);
     auto put = [&](int off, float v) {  // into the tile's rows only
@@ -119,6 +120,13 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
     auto put_if = [&](int off, int next, float v) {
         asm volatile(
             "{ .reg .pred p, q; setp.ne.s32 p, %0, %4; setp.lt.and.u32 q, %0, %1, p; @q st.shared.f32 [%2], %3; }" ::"r"(off),
+            "n"(BV << 10), "r"(zt + off), "f"(v), "r"(next)
+            : "memory");
+    };
+    // the same when the row `next` lies above `off`
+    auto put_above = [&](int off, int next, float v) {
+        asm volatile(
+            "{ .reg .pred p, q; setp.lt.s32 p, %0, %4; setp.lt.and.u32 q, %0, %1, p; @q st.shared.f32 [%2], %3; }" ::"r"(off),
             "n"(BV << 10), "r"(zt + off), "f"(v), "r"(next)
             : "memory");
     };
@@ -144,18 +152,15 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int off = (int)(__float_as_uint(h ? m2.y : m2.x) << 10);
-                    if (!TALL) {
-                        put_if(open, off, acc);
-                        acc = off != open ? acc1 : acc;
-                        acc1 = off != open ? 0.f : acc1;
-                        open = off;
-                    } else {
-                        for (; open < off; open += 1 << 10) {
-                            put(open, acc);
-                            acc = acc1;
-                            acc1 = 0.f;
-                        }
+                    put_if(open, off, acc);
+                    if (TALL) {  // the centre may pass rows
+                        const int next = open + (1 << 10);
+                        put_above(next, off, acc1);
+                        acc1 = off > next ? 0.f : acc1;
                     }
+                    acc = off != open ? acc1 : acc;
+                    acc1 = off != open ? 0.f : acc1;
+                    open = off;
                     acc += h ? own2.y : own2.x;
                     acc1 += h ? up2.y : up2.x;
                 }
