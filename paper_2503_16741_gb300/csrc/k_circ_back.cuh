@@ -193,13 +193,22 @@ __device__ __forceinline__ void filter_rows(const BackCtx<NT> &X, int t, const T
 // 5: than four; 9: than eight).  Row buffer: at most ZT sv + 2 rows with
 // sv < NX - 1, and the NX rows after them that the last voxel may look at with
 // a weight of zero, or of the order of rounding.
-__host__ __device__ constexpr int back_rows(int ZT, int NX) { return ZT * (NX - 1) + 2 + NX; }
+// Voxel-driven, voxels of two rows and more (NX > 3): most of the rows between two
+// voxels' centres are read by neither, so none is filtered beforehand; each voxel
+// filters its own two, and the buffer holds the chunk's sums alone (16 voxels to a
+// thread where that leaves the chip a wave of warps, else 4).  342^2 x 292 / 95 views /
+// 531 x 2056 FP16: every row filtered 20.5 ms, so 9.1.
+__host__ __device__ constexpr bool back_point(int KIND, int NX) { return KIND == BK_VOX && NX > 3; }
+__host__ __device__ constexpr int back_rows(int KIND, int ZT, int NX) {
+    return back_point(KIND, NX) ? ZT : ZT * (NX - 1) + 2 + NX;
+}
 
 template <typename TIn, int KIND, bool CURVED, bool RECON, int NT, int NX, int ZT>
 __global__ void __launch_bounds__(kThreads, 4)
 circ_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sino, void *__restrict__ vol, int out_t,
           int patches_x, int patches, int C, int nzb, int S) {
-    constexpr int NR = back_rows(ZT, NX);
+    constexpr int NR = back_rows(KIND, ZT, NX);
+    constexpr bool POINT = back_point(KIND, NX);
     static_assert(NR >= ZT, "the row buffer also holds the chunk's sums");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BackCtx<NT> *ctx = reinterpret_cast<BackCtx<NT> *>(smem_raw);          // [2]
@@ -264,10 +273,11 @@ circ_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ si
                         lo -= ef;
                         n = (int)ceilf(fmaf(sv, (float)len, lo - 0.5f)) + 1;
                     }
-                    n = min(max(n, 0), NR - NX);
+                    n = min(max(n, 0), POINT ? NR : NR - NX);
                 }
                 const TIn *yp = ys + (size_t)(v0 + vv) * vstride + as;
-                if constexpr (decltype(own)::value) {
+                if constexpr (POINT) {
+                } else if constexpr (decltype(own)::value) {
                     for (int r = 0; r < n; ++r)
                         Rs[r * kThreads + tid] = B + r >= 0 && B + r < g.nv ? own_row(X, t, yp + (size_t)(B + r) * g.nu) : 0.f;
                 } else if (B >= 0 && B + n <= g.nv && !one) {
@@ -308,8 +318,10 @@ circ_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ si
                         rw[0] = R;
                     }
                 }
+                if constexpr (!POINT) {
 #pragma unroll
-                for (int q = 0; q < NX; ++q) Rs[(n + q) * kThreads + tid] = 0.f;  // (read with weight zero)
+                    for (int q = 0; q < NX; ++q) Rs[(n + q) * kThreads + tid] = 0.f;  // (read with weight zero)
+                }
                 // ---- sweep: voxel kk's lower edge (VOX: centre) lies at p = lo + kk sv rows
                 // from row 0's centre (VOX: upper edge); adding 1.5 2^23 rounds p to its row
                 // e and leaves e in the low bits, which shifted by 10 are the row's offset
@@ -334,7 +346,17 @@ circ_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ si
                     const char *ra = rp + (int)(__float_as_uint(m2.x) << 10), *rb = rp + (int)(__float_as_uint(m2.y) << 10);
                     auto row = [](const char *r, int q) { return *reinterpret_cast<const float *>(r + q * 1024); };
                     float2 s2;
-                    if (KIND == BK_VOX) {  // between rows e and e + 1: d and 1 - d
+                    if constexpr (POINT) {
+                        auto at = [&](const char *r, int q) {  // that row, filtered here
+                            const int b = B + (int)((r - rp) >> 10) + q;
+                            if ((unsigned)b >= (unsigned)g.nv) return 0.f;
+                            const TIn *y = yp + (size_t)b * g.nu;
+                            return fmaf(X.F[1][t], ld(y, one ? 0 : 1), X.F[0][t] * ld(y, 0));
+                        };
+                        s2 = __fmul2_rn(d2, make_float2(at(ra, 0), at(rb, 0)));
+                        s2 = __ffma2_rn(__fadd2_rn(make_float2(1.f, 1.f), make_float2(-d2.x, -d2.y)),
+                                        make_float2(at(ra, 1), at(rb, 1)), s2);
+                    } else if (KIND == BK_VOX) {  // between rows e and e + 1: d and 1 - d
                         s2 = __fmul2_rn(d2, make_float2(row(ra, 0), row(rb, 0)));
                         s2 = __ffma2_rn(__fadd2_rn(make_float2(1.f, 1.f), make_float2(-d2.x, -d2.y)),
                                         make_float2(row(ra, 1), row(rb, 1)), s2);
@@ -414,7 +436,7 @@ cudaError_t circ_back_go(const CtGrid &g, const CtView *views, const TIn *src, v
     const int ngrp = (patches + G - 1) / G;
     const int npass = (g.nview + 8 / G - 1) / (8 / G);
     const int S = view_split((long long)patches * nch, npass);
-    const size_t smem = 2 * sizeof(BackCtx<NT>) + sizeof(float) * back_rows(ZT, NX) * kThreads;
+    const size_t smem = 2 * sizeof(BackCtx<NT>) + sizeof(float) * back_rows(KIND, ZT, NX) * kThreads;
     auto kern = circ_back<TIn, KIND, CURVED, RECON, NT, NX, ZT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -438,7 +460,12 @@ cudaError_t circ_back_nx(const CtGrid &g, const CtView *views, const TIn *src, v
     // rows per voxel sv <= 2 max_m_sf_v
     if (g.max_m_sf_v < 0.5f) return circ_back_go<TIn, KIND, CURVED, RECON, NT, 2, 16>(g, views, src, out, out_t, batch, st);
     if (g.max_m_sf_v < 1.f) return circ_back_go<TIn, KIND, CURVED, RECON, NT, 3, 16>(g, views, src, out, out_t, batch, st);
-    if (g.max_m_sf_v < 2.f) return circ_back_go<TIn, KIND, CURVED, RECON, NT, 5, 8>(g, views, src, out, out_t, batch, st);
+    if constexpr (KIND == BK_VOX) {
+        if ((long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4) * ((g.nz + 15) / 16) >= 152 * 32)
+            return circ_back_go<TIn, KIND, CURVED, RECON, NT, 9, 16>(g, views, src, out, out_t, batch, st);
+    } else if (g.max_m_sf_v < 2.f) {
+        return circ_back_go<TIn, KIND, CURVED, RECON, NT, 5, 8>(g, views, src, out, out_t, batch, st);
+    }
     return circ_back_go<TIn, KIND, CURVED, RECON, NT, 9, 4>(g, views, src, out, out_t, batch, st);
 }
 
