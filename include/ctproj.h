@@ -28,10 +28,14 @@
  *     batch x nview x nv x nu floats (non-circular CT_DD only when its
  *     footprints fit the footprint kernels, at most 8 cells by 4 rows);
  *   ct_forward with CT_SF, CT_DD, CT_SF_TT or CT_RAY (cone beam) and with
- *     CT_VOXEL (circular cone beam): a reordered copy of the volume, batch x
- *     nz x ny x nx elements of in_t; but for CT_RAY, in circular geometry with nz rounded up to a
- *     multiple of 4, twice that for CT_SF, CT_DD and CT_VOXEL, and none below 4
- *     slices (skipped, at some speed, when it cannot be had).
+ *     CT_VOXEL (circular cone beam): reordered copies of the volume, batch x nz x
+ *     ny x nx elements of in_t each: one, or two for CT_SF, CT_DD and CT_VOXEL in
+ *     circular geometry when the views' central rays run more along x in some and
+ *     more along y in others.  In circular geometry nz counts rounded up to a
+ *     multiple of 4 (but for CT_RAY), and there is no copy below 4 slices or for
+ *     the smallest calls; CT_RAY needs one only where rays run along x.  The
+ *     copies change no result: a forward that cannot have two takes one, and then
+ *     none, at some speed.
  * ct_workspace_bytes gives that size for a call; ct_workspace_limit caps
  * what the pool keeps once calls have returned it.
  * Results are deterministic: no atomics, fixed summation order.

@@ -194,6 +194,7 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     g->du = d->du;
     g->dv = two_d ? 1.0 : d->dv;
     const bool curved = d->det == CT_DET_CURVED;
+    int main_axes = 0, ray_x = 0;
     g->host_views.resize(d->nview);
     const std::vector<double> dbeta = recon_dbetas(d, P);
 
@@ -242,6 +243,23 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
         V.Cv = (float)(0.5 * (g->nv - 1) - h0 / g->dv);
         V.D = (float)D;
         V.main_y = std::fabs(cs.y) >= std::fabs(cs.x) ? 1 : 0;
+        main_axes |= V.main_y ? 1 : 2;
+        {
+            // Do all rays run more along y than along x (in voxels)?  With e = y dx -+ x dy of
+            // the direction, affine over a flat detector and a sinusoid over an arc of less than
+            // half a turn, it is enough that they do at the corners, all in the same sense.
+            double lo = 1e300, hi = -1e300;  // least of y - |x| and greatest of y + |x|, by length
+            for (int q = 0; q < 4; ++q) {
+                const double u = ((q & 1 ? g->nu - 1 : 0) - (double)V.Cu) * g->du, w = ((q & 2 ? g->nv - 1 : 0) - (double)V.Cv) * g->dv;
+                const Vec3 r = (curved ? D * std::cos(u / D) : D) * n + (curved ? D * std::sin(u / D) : u) * eu + w * ev;
+                const double x = std::fabs(r.x / g->dx) / norm(r), y = r.y / g->dy / norm(r);
+                lo = std::min(lo, y - x);
+                hi = std::max(hi, y + x);
+            }
+            const double tiny = 1e-5 / g->dy;  // (the kernel decides in single precision)
+            const bool wide = curved && (g->nu - 1) * g->du >= 3.1 * D;
+            if (wide || !(lo > tiny || hi < -tiny)) ray_x = 1;
+        }
         const double R = -dot(s, n);  // recon mode: source to rotation centre along n
         V.rc_R = (float)R;
         const double db = dbeta[v];
@@ -332,6 +350,8 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
     G.max_m_dd_u = 0.f;
     G.max_m_sf_v = 0.f;
     G.max_m_tt_v = 0.f;
+    G.axes = main_axes;
+    G.ray_x = ray_x;
     G.nc_tile = G.nc_gather = 0;
     for (const CtView &V : g->host_views) {
         G.max_m_sf_u = std::max(G.max_m_sf_u, V.m_sf_u);
@@ -462,7 +482,7 @@ ct_status ct_back_acc(const ct_geometry *g, ct_projector proj, ct_mode mode, ct_
 }
 
 // Pooled workspace of one projection call, by the same rules the launchers
-// follow (k_sf.cu, k_nc_fwd.cu, k_nc_back.cu, k_ray.cu).
+// follow (k_circ_fwd_f32.cu, k_sf.cu, k_nc_fwd.cu, k_nc_back.cu, k_ray.cu).
 static size_t workspace_rule(int dir, const ct_geometry *g, ct_projector proj, ct_mode mode, ct_dtype in_t,
                              int batch) {
     const CtGrid &G = g->grid;
@@ -476,7 +496,7 @@ static size_t workspace_rule(int dir, const ct_geometry *g, ct_projector proj, c
     if (dir == 0) {
         switch (proj) {
         case CT_VOXEL: return ctp::circ_fwd_fits(G, ctp::BK_VOX, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;
-        case CT_RAY: return G.is2d ? 0 : vox * isz;
+        case CT_RAY: return G.is2d || !G.ray_x ? 0 : vox * isz;
         case CT_DD:
             if (nc) return ctp::nc_footprint_fits(G, 1) ? vox * isz : 0;
             return ctp::circ_fwd_fits(G, ctp::BK_DD, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;

@@ -55,8 +55,7 @@ bool circ_back_fits(const CtGrid &g, int kind);
 cudaError_t launch_circ_back(int kind, bool recon, const CtGrid &g, const CtView *views, int in_t, const void *in,
                              int out_t, void *out, int batch, cudaStream_t st);
 // circular cone-beam forward (k_circ_fwd.cuh) of SF-TR, DD and voxel-driven
-// (kind: BackKind) for footprints of at most 8 cells; cudaErrorMemoryAllocation
-// when its copies of the volume (circ_fwd_workspace bytes) cannot be had
+// (kind: BackKind) for footprints of at most 8 cells
 size_t circ_fwd_workspace(const CtGrid &g, int batch, int elem_bytes);
 bool circ_fwd_fits(const CtGrid &g, int kind, int batch);
 cudaError_t launch_circ_fwd(int kind, const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,

@@ -57,6 +57,8 @@ struct CtGrid {
     float max_m_dd_u;  // largest per-view DD boundary bound (cells)
     float max_m_sf_v;  // largest per-view axial half-height bound (rows)
     float max_m_tt_v;  // largest per-view SF-TT axial bound (rows)
+    int axes;          // main axes of the views: bit 0 some view's is y, bit 1 some view's is x
+    int ray_x;         // some view may have rays that run mainly along x
     int nc_tile;       // non-circular: some view has CtView::nc_tile set,
     int nc_gather;     // some view has not
     float alpha, beta; // output epilogue: out = alpha * result + beta * out

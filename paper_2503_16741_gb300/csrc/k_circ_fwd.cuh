@@ -47,6 +47,12 @@ inline long long circ_fwd_ctas(const CtGrid &g, int cells, int batch) {
     return (long long)((g.nu + cells - 1) / cells) * ((g.nv + 63) / 64) * g.nview * batch;
 }
 constexpr long long kFwdWave = 3 * 152;
+// What the kernel reads: the copies (nzp > 0: slices of one; see circ_fwd) or, nzp = 0,
+// the volume in place, which gives the same results, slower where the copies pay
+struct FwdVolume {
+    const void *y, *x;
+    int nzp;
+};
 // Volumes of at most 32^3 voxels in calls of few CTAs are read in place: the copies
 // would cost such a call an allocation and a launch, a third of its time.
 inline bool circ_fwd_direct(const CtGrid &g, int batch) {
@@ -213,11 +219,12 @@ __device__ __forceinline__ void circ_walk(const CtGrid &g, const TIn *__restrict
 
 // CTA = CELLS cells x BV rows, RPT rows to a thread, NG threads to a cell.
 // (BV = 64: 3 blocks per SM by shared memory and 80 registers; 32 x 32: 4 at 64)
-// DIRECT: the volume itself instead of its copies.
+// vol_y, vol_x: the copies for the views whose main axis is y and x; null: not these
+// views.  DIRECT: the volume itself instead.
 template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL, bool DIRECT>
 __global__ void __launch_bounds__(256, BV == 64 ? 3 : 4)
-circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, int nzp, void *__restrict__ sino,
-         int out_t, int tiles_u, int tiles_v) {
+circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol_y, const TIn *__restrict__ vol_x, int nzp,
+         void *__restrict__ sino, int out_t, int tiles_u, int tiles_v) {
     constexpr int NG = 256 / CELLS, RPT = BV / NG;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CircFwdSmem<BV, NT> &S = *reinterpret_cast<CircFwdSmem<BV, NT> *>(smem_raw);
@@ -233,13 +240,15 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
     const int a = A0 + ac;
     const CtView &V = views[v];
     const int main_y = V.main_y;
+    const TIn *xz = main_y ? vol_y : vol_x;
+    if (!xz) return;  // (whole CTA)
     const SlabCoef sc = slab_coef(V, main_y);
     // search half widths: footprint bound + half a cell, or the hat's one cell
     const float mu = KIND == BK_VOX ? 1.f + kSearchPad : (KIND == BK_DD ? V.m_dd_u : V.m_sf_u) + 0.5f + kSearchPad;
     const float mv = KIND == BK_VOX ? 1.f + kSearchPad : V.m_sf_v + 0.5f + kSearchPad;
     const int nslab = main_y ? g.ny : g.nx, nlat = main_y ? g.nx : g.ny;
     // the copy whose columns are adjacent along the view's lateral axis
-    const TIn *xz = vol + (DIRECT ? (size_t)bt * g.nz : ((size_t)bt * 2 + (main_y ? 0 : 1)) * nzp) * g.nx * g.ny;
+    xz += (size_t)bt * (DIRECT ? g.nz : nzp) * g.nx * g.ny;
     // the two lines of constant u that bound the cell's reach: lateral index = p + s slab
     float p1, s1, p2, s2;
     {
@@ -402,7 +411,7 @@ circ_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol
 // ------------------------------------------------------------ launchers
 namespace {
 template <typename TIn, int KIND, bool CURVED, int CELLS, int BV, int NT, bool TALL, bool DIRECT = false>
-cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *x, int nzp, void *out, int out_t, int batch,
+cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const FwdVolume &x, void *out, int out_t, int batch,
                         cudaStream_t st) {
     const int tiles_u = (g.nu + CELLS - 1) / CELLS, tiles_v = (g.nv + BV - 1) / BV;
     const size_t smem = sizeof(CircFwdSmem<BV, NT>);
@@ -410,7 +419,7 @@ cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *x, int 
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((unsigned)((size_t)tiles_u * tiles_v * g.nview * batch)), dim3(32, 8), smem, st>>>(
-        g, views, x, nzp, out, out_t, tiles_u, tiles_v);
+        g, views, static_cast<const TIn *>(x.y), static_cast<const TIn *>(x.x), x.nzp, out, out_t, tiles_u, tiles_v);
     return cudaGetLastError();
 }
 
@@ -432,63 +441,64 @@ cudaError_t circ_fwd_go(const CtGrid &g, const CtView *views, const TIn *x, int 
 // view, up to twice the time for a few.)  Voxels that may cover whole rows have a walk
 // that spills at 64 x 64 (183^2 x 157 / 231 views DD 3.7 -> 4.2 ms).
 template <typename TIn, int KIND, bool CURVED, int NT, bool TALL>
-cudaError_t circ_fwd_rpt(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
+cudaError_t circ_fwd_rpt(const CtGrid &g, const CtView *views, const FwdVolume &x, void *out, int out_t, int batch,
                          cudaStream_t st) {
-    // (TALL everywhere: one kernel serves either height of voxels in small calls)
-    const bool direct = circ_fwd_direct(g, batch);
-    if (g.nv <= 8)
-        return direct ? circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true, true>(g, views, xZ, nzp, out, out_t, batch, st)
-                      : circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true>(g, views, xZ, nzp, out, out_t, batch, st);
-    if (direct) return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, true, true>(g, views, xZ, nzp, out, out_t, batch, st);
+    // (TALL everywhere: one kernel serves either height of voxels in small calls and in place)
+    if (x.nzp == 0) {
+        if (g.nv <= 8) return circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true, true>(g, views, x, out, out_t, batch, st);
+        if (circ_fwd_ctas(g, 32, batch) < kFwdWave)
+            return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, true, true>(g, views, x, out, out_t, batch, st);
+        return circ_fwd_go<TIn, KIND, CURVED, 32, 64, NT, true, true>(g, views, x, out, out_t, batch, st);
+    }
+    if (g.nv <= 8) return circ_fwd_go<TIn, KIND, CURVED, 32, 8, NT, true>(g, views, x, out, out_t, batch, st);
     if (circ_fwd_ctas(g, 16, batch) < kFwdWave / 2)
-        return circ_fwd_go<TIn, KIND, CURVED, 8, 64, NT, true>(g, views, xZ, nzp, out, out_t, batch, st);
+        return circ_fwd_go<TIn, KIND, CURVED, 8, 64, NT, true>(g, views, x, out, out_t, batch, st);
     if (circ_fwd_ctas(g, 32, batch) < kFwdWave)
-        return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
-    if (g.nv <= 32) return circ_fwd_go<TIn, KIND, CURVED, 32, 32, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+        return circ_fwd_go<TIn, KIND, CURVED, 16, 64, NT, TALL>(g, views, x, out, out_t, batch, st);
+    if (g.nv <= 32) return circ_fwd_go<TIn, KIND, CURVED, 32, 32, NT, TALL>(g, views, x, out, out_t, batch, st);
     if constexpr (!TALL)
         if (circ_fwd_ctas(g, 64, batch) >= 2 * kFwdWave)
-            return circ_fwd_go<TIn, KIND, CURVED, 64, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
-    return circ_fwd_go<TIn, KIND, CURVED, 32, 64, NT, TALL>(g, views, xZ, nzp, out, out_t, batch, st);
+            return circ_fwd_go<TIn, KIND, CURVED, 64, 64, NT, TALL>(g, views, x, out, out_t, batch, st);
+    return circ_fwd_go<TIn, KIND, CURVED, 32, 64, NT, TALL>(g, views, x, out, out_t, batch, st);
 }
 
 template <typename TIn, int KIND, bool CURVED, int NT>
-cudaError_t circ_fwd_nx(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
+cudaError_t circ_fwd_nx(const CtGrid &g, const CtView *views, const FwdVolume &x, void *out, int out_t, int batch,
                         cudaStream_t st) {
     // rows per voxel: at most 2 max_m_sf_v
-    if (g.max_m_sf_v < 0.5f) return circ_fwd_rpt<TIn, KIND, CURVED, NT, false>(g, views, xZ, nzp, out, out_t, batch, st);
-    return circ_fwd_rpt<TIn, KIND, CURVED, NT, true>(g, views, xZ, nzp, out, out_t, batch, st);
+    if (g.max_m_sf_v < 0.5f) return circ_fwd_rpt<TIn, KIND, CURVED, NT, false>(g, views, x, out, out_t, batch, st);
+    return circ_fwd_rpt<TIn, KIND, CURVED, NT, true>(g, views, x, out, out_t, batch, st);
 }
 
 template <typename TIn, int KIND, bool CURVED>
-cudaError_t circ_fwd_nt(const CtGrid &g, const CtView *views, const TIn *xZ, int nzp, void *out, int out_t, int batch,
+cudaError_t circ_fwd_nt(const CtGrid &g, const CtView *views, const FwdVolume &x, void *out, int out_t, int batch,
                         cudaStream_t st) {
     if constexpr (KIND == BK_VOX) {
-        return circ_fwd_nx<TIn, KIND, CURVED, 2>(g, views, xZ, nzp, out, out_t, batch, st);
+        return circ_fwd_nx<TIn, KIND, CURVED, 2>(g, views, x, out, out_t, batch, st);
     } else {
         // cells that a footprint of half width m may meet: ceil(2 m) + 1
         const float m = KIND == BK_DD ? g.max_m_dd_u : g.max_m_sf_u;
-        if (m <= 1.f) return circ_fwd_nx<TIn, KIND, CURVED, 3>(g, views, xZ, nzp, out, out_t, batch, st);
-        if (m <= 1.5f) return circ_fwd_nx<TIn, KIND, CURVED, 4>(g, views, xZ, nzp, out, out_t, batch, st);
-        if (m <= 2.5f) return circ_fwd_nx<TIn, KIND, CURVED, 6>(g, views, xZ, nzp, out, out_t, batch, st);
-        return circ_fwd_nx<TIn, KIND, CURVED, 8>(g, views, xZ, nzp, out, out_t, batch, st);
+        if (m <= 1.f) return circ_fwd_nx<TIn, KIND, CURVED, 3>(g, views, x, out, out_t, batch, st);
+        if (m <= 1.5f) return circ_fwd_nx<TIn, KIND, CURVED, 4>(g, views, x, out, out_t, batch, st);
+        if (m <= 2.5f) return circ_fwd_nx<TIn, KIND, CURVED, 6>(g, views, x, out, out_t, batch, st);
+        return circ_fwd_nx<TIn, KIND, CURVED, 8>(g, views, x, out, out_t, batch, st);
     }
 }
 
 template <typename TIn>
-cudaError_t circ_fwd_kind(int kind, const CtGrid &g, const CtView *views, const void *xZ, int nzp, void *out,
+cudaError_t circ_fwd_kind(int kind, const CtGrid &g, const CtView *views, const FwdVolume &x, void *out,
                           int out_t, int batch, cudaStream_t st) {
-    const TIn *src = static_cast<const TIn *>(xZ);
     const bool curved = g.variant == GEO_CIRC_CURVED;
     switch (kind) {
     case BK_SF:
-        return curved ? circ_fwd_nt<TIn, BK_SF, true>(g, views, src, nzp, out, out_t, batch, st)
-                      : circ_fwd_nt<TIn, BK_SF, false>(g, views, src, nzp, out, out_t, batch, st);
+        return curved ? circ_fwd_nt<TIn, BK_SF, true>(g, views, x, out, out_t, batch, st)
+                      : circ_fwd_nt<TIn, BK_SF, false>(g, views, x, out, out_t, batch, st);
     case BK_DD:
-        return curved ? circ_fwd_nt<TIn, BK_DD, true>(g, views, src, nzp, out, out_t, batch, st)
-                      : circ_fwd_nt<TIn, BK_DD, false>(g, views, src, nzp, out, out_t, batch, st);
+        return curved ? circ_fwd_nt<TIn, BK_DD, true>(g, views, x, out, out_t, batch, st)
+                      : circ_fwd_nt<TIn, BK_DD, false>(g, views, x, out, out_t, batch, st);
     default:
-        return curved ? circ_fwd_nt<TIn, BK_VOX, true>(g, views, src, nzp, out, out_t, batch, st)
-                      : circ_fwd_nt<TIn, BK_VOX, false>(g, views, src, nzp, out, out_t, batch, st);
+        return curved ? circ_fwd_nt<TIn, BK_VOX, true>(g, views, x, out, out_t, batch, st)
+                      : circ_fwd_nt<TIn, BK_VOX, false>(g, views, x, out, out_t, batch, st);
     }
 }
 }  // namespace

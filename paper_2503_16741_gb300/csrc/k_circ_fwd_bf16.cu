@@ -4,9 +4,9 @@
 
 namespace ctp {
 
-cudaError_t circ_fwd_bf16(int kind, const CtGrid &g, const CtView *views, const void *xZ, int nzp, void *out, int out_t,
+cudaError_t circ_fwd_bf16(int kind, const CtGrid &g, const CtView *views, const FwdVolume &x, void *out, int out_t,
                          int batch, cudaStream_t st) {
-    return circ_fwd_kind<__nv_bfloat16>(kind, g, views, xZ, nzp, out, out_t, batch, st);
+    return circ_fwd_kind<__nv_bfloat16>(kind, g, views, x, out, out_t, batch, st);
 }
 
 }  // namespace ctp

@@ -412,9 +412,10 @@ cudaError_t ray_launch_t(int dir, const CtGrid &g, const CtView *views, const vo
     const TIn *src = static_cast<const TIn *>(in);
     if (dir == 0) {
         const int tiles_u = (g.nu + 31) / 32;
-        TIn *xT = nullptr;  // (without it, rays along x read strided)
+        TIn *xT = nullptr;  // for rays along x, where there may be some (without it they read strided)
         const long long slices = (long long)g.nz * batch;
-        if (workspace_alloc((void **)&xT, (size_t)g.nx * g.ny * slices * sizeof(TIn), st) != cudaSuccess) {
+        if (!g.ray_x) {
+        } else if (workspace_alloc((void **)&xT, (size_t)g.nx * g.ny * slices * sizeof(TIn), st) != cudaSuccess) {
             cudaGetLastError();
             xT = nullptr;
         } else {

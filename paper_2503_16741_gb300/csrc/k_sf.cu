@@ -1040,8 +1040,8 @@ cudaError_t fp_fwd_stream(const CtGrid &g, const CtView *views, const TIn *src, 
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // SF-TT walks a z-major copy of the volume (pooled workspace), one vector
-    // load per four voxels; without it, and in the other projectors (here only
-    // when that copy could not be had), the walks read strided
+    // load per four voxels; without it, and in the other projectors (sizes that
+    // k_circ_fwd.cuh does not take), the walks read strided
     TIn *xZ = nullptr;
     const int nzp = TT && zmajor_copy_fits(g, batch) ? zmajor_pitch(g) : 0;
     if (nzp) {
@@ -1281,11 +1281,8 @@ cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny,
 
 cudaError_t launch_vx_fwd_circ(const CtGrid &g, const CtView *views, int in_t, const void *in, int out_t,
                                void *out, int batch, cudaStream_t st) {
-    if (circ_fwd_fits(g, BK_VOX, batch)) {
-        const cudaError_t e = launch_circ_fwd(BK_VOX, g, views, in_t, in, out_t, out, batch, st);
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-    }
+    if (circ_fwd_fits(g, BK_VOX, batch))
+        return launch_circ_fwd(BK_VOX, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return vx_fwd_t<float>(g, views, in, out, out_t, batch, st);
     case 1: return vx_fwd_t<__half>(g, views, in, out, out_t, batch, st);
@@ -1327,11 +1324,8 @@ cudaError_t launch_sf(int dir, const CtGrid &g, const CtView *views, int in_t, c
     if (g.variant == GEO_NONCIRC_FLAT && nc_footprint_fits(g, 0))
         return launch_nc(0, dir, g, views, in_t, in, out_t, out, batch, st);
     if (fan_fits(g, FAN_SF, dir)) return launch_fan(FAN_SF, dir, g, views, in_t, in, out_t, out, batch, st);
-    if (dir == 0 && circ_fwd_fits(g, BK_SF, batch)) {
-        const cudaError_t e = launch_circ_fwd(BK_SF, g, views, in_t, in, out_t, out, batch, st);
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-    }
+    if (dir == 0 && circ_fwd_fits(g, BK_SF, batch))
+        return launch_circ_fwd(BK_SF, g, views, in_t, in, out_t, out, batch, st);
     if (dir == 1 && circ_back_fits(g, BK_SF))
         return launch_circ_back(BK_SF, false, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
@@ -1353,11 +1347,8 @@ cudaError_t launch_dd(int dir, const CtGrid &g, const CtView *views, int in_t, c
         }
     }
     if (dir == 0 && fan_fits(g, FAN_DD, 0)) return launch_fan(FAN_DD, 0, g, views, in_t, in, out_t, out, batch, st);
-    if (dir == 0 && circ_fwd_fits(g, BK_DD, batch)) {
-        const cudaError_t e = launch_circ_fwd(BK_DD, g, views, in_t, in, out_t, out, batch, st);
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-    }
+    if (dir == 0 && circ_fwd_fits(g, BK_DD, batch))
+        return launch_circ_fwd(BK_DD, g, views, in_t, in, out_t, out, batch, st);
     switch (in_t) {
     case 0: return dd_launch_t<float>(dir, g, views, in, out, out_t, batch, st);
     case 1: return dd_launch_t<__half>(dir, g, views, in, out, out_t, batch, st);

@@ -73,3 +73,20 @@ def test_workspace_limit_releases_freed_blocks(ct):
     held, _ = ct.workspace_usage()
     assert held == 0
     ct.workspace_limit(1 << 62)
+
+
+def test_only_the_copies_that_the_views_need(ct):
+    """Views whose central rays run along y, along x and along both."""
+    spec = W.scaled(W.circ3d_256(), 64, 45)
+    g = ct.Geometry.from_spec(spec)
+    th = np.asarray(spec.theta)
+    along_y = np.abs(np.cos(th)) > 0.9
+    x = torch.rand(g.vol_shape, device="cuda")
+    one = 4 * 64 ** 3
+    for proj, none in (("sf", one), ("ray", 0)):
+        y = ct.forward(g, x, proj)
+        for views, want in ((np.flatnonzero(along_y), none), (np.flatnonzero(np.abs(np.sin(th)) > 0.9), one)):
+            s = g.subset(np.tile(views, 8))
+            assert ct.workspace_bytes(s, proj, "fwd") == want
+            assert torch.equal(ct.forward(s, x, proj), y[np.tile(views, 8)])
+    assert ct.workspace_bytes(g, "sf", "fwd", batch=4) == 4 * 2 * one
