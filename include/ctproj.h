@@ -35,7 +35,7 @@
  *     multiple of 4 (but for CT_RAY), and there is no copy below 4 slices or for
  *     the smallest calls; CT_RAY needs one only where rays run along x.  The
  *     copies change no result: a forward that cannot have two takes one, and then
- *     none, at some speed.
+ *     none, at some speed (ct_forward_within caps them).
  * ct_workspace_bytes gives that size for a call; ct_workspace_limit caps
  * what the pool keeps once calls have returned it.
  * Results are deterministic: no atomics, fixed summation order.
@@ -208,6 +208,14 @@ ct_status ct_back_acc(const ct_geometry *geom, ct_projector proj, ct_mode mode,
                       ct_dtype in_t, const void *sino, ct_dtype out_t, void *vol,
                       int batch, float alpha, float beta, void *cuda_stream);
 
+/* ct_forward_acc with at most workspace_max bytes of pooled workspace, for
+ * callers that account for device memory: a forward's copies of the volume
+ * are left out, one by one, until the rest fits.  The result is that of
+ * ct_forward_acc bit for bit. */
+ct_status ct_forward_within(const ct_geometry *geom, ct_projector proj, ct_mode mode,
+                            ct_dtype in_t, const void *vol, ct_dtype out_t, void *sino,
+                            int batch, float alpha, float beta, size_t workspace_max, void *cuda_stream);
+
 /* Distance-driven backprojection (as ct_back with CT_DD, CT_MODE_PROJ) that
  * allocates no device memory.  The paper has no counterpart: this entry point
  * exists for callers that cannot call cudaMalloc or take memory from a pool
@@ -262,6 +270,11 @@ ct_status ct_ramp_filter(const ct_geometry *geom, ct_dtype in_t, const void *sin
  * enums, a direction other than 0 / 1 or batch < 1. */
 ct_status ct_workspace_bytes(const ct_geometry *geom, ct_projector proj, ct_mode mode, int direction,
                              ct_dtype in_t, int batch, size_t *bytes);
+
+/* The workspace (bytes) that ct_forward_within takes in CT_MODE_PROJ under
+ * workspace_max; arguments and errors as for ct_workspace_bytes. */
+ct_status ct_forward_workspace_within(const ct_geometry *geom, ct_projector proj, ct_dtype in_t, int batch,
+                                      size_t workspace_max, size_t *bytes);
 
 /* Caps the bytes the current device's pool keeps once calls have returned
  * their workspace: blocks above `bytes` go back to the device at the next

@@ -88,6 +88,10 @@ def load():
         lib.ct_back_acc.argtypes = sig_acc
         lib.ct_forward_acc.restype = C.c_int
         lib.ct_back_acc.restype = C.c_int
+        lib.ct_forward_within.argtypes = sig[:-1] + [C.c_float, C.c_float, C.c_size_t, C.c_void_p]
+        lib.ct_forward_within.restype = C.c_int
+        lib.ct_forward_workspace_within.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_size_t, P(C.c_size_t)]
+        lib.ct_forward_workspace_within.restype = C.c_int
         lib.ct_back_dd_noalloc.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p,
                                            C.c_int, C.c_void_p]
         lib.ct_back_dd_noalloc.restype = C.c_int
@@ -235,15 +239,20 @@ def _check_tensor(t: torch.Tensor, what: str):
 
 
 def forward_into(geom: Geometry, x: torch.Tensor, y: torch.Tensor, projector: str = "sf",
-                 mode: str = "proj", stream=None) -> torch.Tensor:
-    """y = A x into a preallocated sinogram tensor (Sec. 2.3, Eq. 1)."""
+                 mode: str = "proj", stream=None, max_workspace: Optional[int] = None) -> torch.Tensor:
+    """y = A x into a preallocated sinogram tensor (Sec. 2.3, Eq. 1).
+    `max_workspace`: bytes of pooled workspace that the call may take
+    (ct_forward_within; the result does not depend on it)."""
     _check_tensor(x, "volume")
     _check_tensor(y, "sinogram")
     b = _batch_of(x, geom.vol_shape, "volume")
     if _batch_of(y, geom.sino_shape, "sinogram") != b:
         raise ValueError("volume and sinogram batch sizes differ")
-    _check(load().ct_forward(geom.handle, PROJECTORS[projector], MODES[mode], DTYPES[x.dtype],
-                             x.data_ptr(), DTYPES[y.dtype], y.data_ptr(), b, _stream_ptr(stream)))
+    args = (geom.handle, PROJECTORS[projector], MODES[mode], DTYPES[x.dtype], x.data_ptr(), DTYPES[y.dtype], y.data_ptr(), b)
+    if max_workspace is None:
+        _check(load().ct_forward(*args, _stream_ptr(stream)))
+    else:
+        _check(load().ct_forward_within(*args, 1.0, 0.0, int(max_workspace), _stream_ptr(stream)))
     return y
 
 
@@ -261,16 +270,21 @@ def back_into(geom: Geometry, y: torch.Tensor, x: torch.Tensor, projector: str =
 
 
 def forward_acc(geom: Geometry, x: torch.Tensor, y: torch.Tensor, alpha: float, beta: float,
-                projector: str = "sf", mode: str = "proj", stream=None) -> torch.Tensor:
-    """y <- alpha A x + beta y, in place (y's dtype is the storage type)."""
+                projector: str = "sf", mode: str = "proj", stream=None,
+                max_workspace: Optional[int] = None) -> torch.Tensor:
+    """y <- alpha A x + beta y, in place (y's dtype is the storage type);
+    `max_workspace` as for forward_into."""
     _check_tensor(x, "volume")
     _check_tensor(y, "sinogram")
     b = _batch_of(x, geom.vol_shape, "volume")
     if _batch_of(y, geom.sino_shape, "sinogram") != b:
         raise ValueError("volume and sinogram batch sizes differ")
-    _check(load().ct_forward_acc(geom.handle, PROJECTORS[projector], MODES[mode], DTYPES[x.dtype],
-                                 x.data_ptr(), DTYPES[y.dtype], y.data_ptr(), b, float(alpha),
-                                 float(beta), _stream_ptr(stream)))
+    args = (geom.handle, PROJECTORS[projector], MODES[mode], DTYPES[x.dtype], x.data_ptr(), DTYPES[y.dtype], y.data_ptr(), b,
+            float(alpha), float(beta))
+    if max_workspace is None:
+        _check(load().ct_forward_acc(*args, _stream_ptr(stream)))
+    else:
+        _check(load().ct_forward_within(*args, int(max_workspace), _stream_ptr(stream)))
     return y
 
 
@@ -348,6 +362,16 @@ def workspace_bytes(geom: Geometry, projector: str, direction: str, dtype: torch
     out = C.c_size_t(0)
     _check(load().ct_workspace_bytes(geom.handle, PROJECTORS[projector], MODES[mode],
                                      {"fwd": 0, "back": 1}[direction], DTYPES[dtype], int(batch), C.byref(out)))
+    return int(out.value)
+
+
+def forward_workspace_within(geom: Geometry, projector: str, max_workspace: int,
+                             dtype: torch.dtype = torch.float32, batch: int = 1) -> int:
+    """Pooled workspace (bytes) a forward takes under `max_workspace`
+    (ct_forward_workspace_within)."""
+    out = C.c_size_t(0)
+    _check(load().ct_forward_workspace_within(geom.handle, PROJECTORS[projector], DTYPES[dtype], int(batch),
+                                              int(max_workspace), C.byref(out)))
     return int(out.value)
 
 

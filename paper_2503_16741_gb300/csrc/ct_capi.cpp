@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <new>
 #include <string>
@@ -346,6 +347,7 @@ ct_status ct_geometry_create(const ct_geometry_desc *d, ct_geometry **out) {
                                         : (curved ? ctp::GEO_CIRC_CURVED : ctp::GEO_CIRC_FLAT);
     G.alpha = 1.f;
     G.beta = 0.f;
+    G.copy_max = SIZE_MAX;
     G.max_m_sf_u = 0.f;
     G.max_m_dd_u = 0.f;
     G.max_m_sf_v = 0.f;
@@ -411,7 +413,7 @@ static ct_status check_ptr(const void *p, const char *what) { return ctp::check_
 
 static ct_status project(int dir, const ct_geometry *g, ct_projector proj, ct_mode mode, ct_dtype in_t,
                          const void *in, ct_dtype out_t, void *out, int batch, float alpha, float beta,
-                         void *stream) {
+                         void *stream, size_t copy_max = SIZE_MAX) {
     if (!g) return fail(CT_ERR_INVALID_ARG, "null geometry");
     if (proj < CT_VOXEL || proj > CT_SF_TT) return fail(CT_ERR_INVALID_ARG, "unknown projector");
     if (mode != CT_MODE_PROJ && mode != CT_MODE_RECON) return fail(CT_ERR_INVALID_ARG, "unknown mode");
@@ -443,6 +445,7 @@ static ct_status project(int dir, const ct_geometry *g, ct_projector proj, ct_mo
     CtGrid G = g->grid;
     G.alpha = alpha;
     G.beta = beta;
+    G.copy_max = copy_max;
     cudaError_t e;
     switch (mode == CT_MODE_RECON ? -1 - (int)proj : (int)proj) {
     case -1 - CT_VOXEL: e = ctp::launch_voxel_recon(G, g->dev_views, in_t, in, out_t, out, batch, s); break;
@@ -479,6 +482,12 @@ ct_status ct_forward_acc(const ct_geometry *g, ct_projector proj, ct_mode mode, 
 ct_status ct_back_acc(const ct_geometry *g, ct_projector proj, ct_mode mode, ct_dtype in_t, const void *sino,
                       ct_dtype out_t, void *vol, int batch, float alpha, float beta, void *cuda_stream) {
     return project(1, g, proj, mode, in_t, sino, out_t, vol, batch, alpha, beta, cuda_stream);
+}
+
+ct_status ct_forward_within(const ct_geometry *g, ct_projector proj, ct_mode mode, ct_dtype in_t, const void *vol,
+                            ct_dtype out_t, void *sino, int batch, float alpha, float beta, size_t workspace_max,
+                            void *cuda_stream) {
+    return project(0, g, proj, mode, in_t, vol, out_t, sino, batch, alpha, beta, cuda_stream, workspace_max);
 }
 
 // Pooled workspace of one projection call, by the same rules the launchers
@@ -525,6 +534,17 @@ ct_status ct_workspace_bytes(const ct_geometry *g, ct_projector proj, ct_mode mo
     if (in_t < CT_F32 || in_t > CT_BF16) return fail(CT_ERR_INVALID_ARG, "unknown dtype");
     if (batch < 1) return fail(CT_ERR_INVALID_ARG, "batch must be >= 1");
     *bytes = workspace_rule(direction, g, proj, mode, in_t, batch);
+    return CT_OK;
+}
+
+ct_status ct_forward_workspace_within(const ct_geometry *g, ct_projector proj, ct_dtype in_t, int batch,
+                                      size_t workspace_max, size_t *bytes) {
+    const ct_status st = ct_workspace_bytes(g, proj, CT_MODE_PROJ, 0, in_t, batch, bytes);
+    if (st != CT_OK || *bytes <= workspace_max) return st;
+    // one copy of two, or none
+    const bool halves = g->grid.axes == 3 && (proj == CT_SF || proj == CT_DD || proj == CT_VOXEL) &&
+                        g->grid.variant != ctp::GEO_NONCIRC_FLAT;
+    *bytes = halves && *bytes / 2 <= workspace_max ? *bytes / 2 : 0;
     return CT_OK;
 }
 

@@ -100,6 +100,10 @@ inline bool zmajor_copy_fits(const CtGrid &g, int batch) { return batch <= 65535
 // (memory is kept in the pool between calls, so steady-state calls do not
 // reach the driver's allocator).
 cudaError_t workspace_alloc(void **p, size_t bytes, cudaStream_t st);
+// the same for a reordered copy of the volume, which a forward can do without
+inline cudaError_t workspace_alloc_copy(void **p, size_t bytes, const CtGrid &g, cudaStream_t st) {
+    return bytes > g.copy_max ? cudaErrorMemoryAllocation : workspace_alloc(p, bytes, st);
+}
 cudaError_t workspace_free(void *p, cudaStream_t st);
 // release threshold of the current device's pool (and a trim to it)
 cudaError_t workspace_set_limit(size_t bytes);

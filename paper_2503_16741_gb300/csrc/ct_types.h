@@ -61,6 +61,7 @@ struct CtGrid {
     int ray_x;         // some view may have rays that run mainly along x
     int nc_tile;       // non-circular: some view has CtView::nc_tile set,
     int nc_gather;     // some view has not
+    size_t copy_max;   // bytes that the call's reordered copies of the volume may take
     float alpha, beta; // output epilogue: out = alpha * result + beta * out
 };
 

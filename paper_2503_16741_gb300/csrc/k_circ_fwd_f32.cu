@@ -90,7 +90,7 @@ cudaError_t launch_circ_fwd(int kind, const CtGrid &g, const CtView *views, int 
     char *buf = nullptr;
     int copies = circ_fwd_direct(g, batch) ? 0 : g.axes == 3 ? 2 : 1;
     for (; copies > 0; --copies) {
-        if (workspace_alloc((void **)&buf, one * copies, st) == cudaSuccess) break;
+        if (workspace_alloc_copy((void **)&buf, one * copies, g, st) == cudaSuccess) break;
         cudaGetLastError();
         buf = nullptr;
     }

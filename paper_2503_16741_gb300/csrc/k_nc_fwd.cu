@@ -409,7 +409,7 @@ template <typename TIn, int KIND, int NA, int NB> struct NcFwd {
         // reads contiguous along k; without it the reads are strided
         TIn *xZ = nullptr;
         const size_t n = (size_t)g.nx * g.ny * g.nz * batch;
-        if (workspace_alloc((void **)&xZ, n * sizeof(TIn), st) != cudaSuccess) {
+        if (workspace_alloc_copy((void **)&xZ, n * sizeof(TIn), g, st) != cudaSuccess) {
             cudaGetLastError();
             xZ = nullptr;
         } else if ((e = zmajor_copy(sizeof(TIn), src, xZ, g.nx, g.ny, g.nz, g.nz, batch, st)) != cudaSuccess) {

@@ -415,7 +415,7 @@ cudaError_t ray_launch_t(int dir, const CtGrid &g, const CtView *views, const vo
         TIn *xT = nullptr;  // for rays along x, where there may be some (without it they read strided)
         const long long slices = (long long)g.nz * batch;
         if (!g.ray_x) {
-        } else if (workspace_alloc((void **)&xT, (size_t)g.nx * g.ny * slices * sizeof(TIn), st) != cudaSuccess) {
+        } else if (workspace_alloc_copy((void **)&xT, (size_t)g.nx * g.ny * slices * sizeof(TIn), g, st) != cudaSuccess) {
             cudaGetLastError();
             xT = nullptr;
         } else {

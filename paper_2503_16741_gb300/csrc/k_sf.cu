@@ -1045,7 +1045,7 @@ cudaError_t fp_fwd_stream(const CtGrid &g, const CtView *views, const TIn *src, 
     TIn *xZ = nullptr;
     const int nzp = TT && zmajor_copy_fits(g, batch) ? zmajor_pitch(g) : 0;
     if (nzp) {
-        if (workspace_alloc((void **)&xZ, (size_t)g.nx * g.ny * nzp * batch * sizeof(TIn), st) != cudaSuccess) {
+        if (workspace_alloc_copy((void **)&xZ, (size_t)g.nx * g.ny * nzp * batch * sizeof(TIn), g, st) != cudaSuccess) {
             cudaGetLastError();
             xZ = nullptr;
         } else if ((e = zmajor_copy(sizeof(TIn), src, xZ, g.nx, g.ny, g.nz, nzp, batch, st)) != cudaSuccess) {

@@ -39,11 +39,13 @@ def ls_step_size(geom: Geometry, projector: str, **kw) -> float:
 
 def ls_gradient_descent(geom: Geometry, y: torch.Tensor, projector: str, steps: int,
                         lr: Optional[float] = None, x0: Optional[torch.Tensor] = None,
-                        stream=None, work: Optional[torch.Tensor] = None) -> torch.Tensor:
+                        stream=None, work: Optional[torch.Tensor] = None,
+                        max_workspace: Optional[int] = None) -> torch.Tensor:
     """`steps` gradient steps on 1/2 ||A x - y||^2 from x0 (zeros by default).
     y: (..., nview, [nv,] nu); returns x with y's batch shape and dtype.  The
     residual A x - y is kept in FP32 whatever y's storage type (in half
-    storage the difference of two close values would lose its digits)."""
+    storage the difference of two close values would lose its digits).
+    `max_workspace`: see binding.forward_into."""
     if lr is None:
         lr = ls_step_size(geom, projector)
     lead = y.shape[:-len(geom.sino_shape)]
@@ -54,7 +56,7 @@ def ls_gradient_descent(geom: Geometry, y: torch.Tensor, projector: str, steps: 
         r = torch.empty(y.shape, dtype=torch.float32, device=y.device) if work is None else work
         for _ in range(steps):
             r.copy_(y)
-            forward_acc(geom, x, r, 1.0, -1.0, projector, stream=s)
+            forward_acc(geom, x, r, 1.0, -1.0, projector, stream=s, max_workspace=max_workspace)
             back_acc(geom, r, x, -lr, 1.0, projector, stream=s)
     return x
 

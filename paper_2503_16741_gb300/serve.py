@@ -14,7 +14,8 @@ may carry a device tensor and ask for its result on the device, so volumes
 and sinograms stay resident too.  Admission counts every byte a request
 holds on the device while it runs: its input, output and temporaries and the
 library's pooled workspace (ct_workspace_bytes), whose pool is capped at the
-budget.
+budget.  A request that fits the budget only without some of the forward's
+copies of the volume runs without them.
 
 The scheduler is independent of the device: `Scheduler` drives an
 `Executor` (launch a group, poll it, collect results).  `GpuExecutor` runs
@@ -116,8 +117,17 @@ class Executor:
         """Device bytes the request holds while it runs (admission)."""
         return request_bytes(req)
 
+    def fit_bytes(self, req: Request, budget: int) -> int:
+        """request_bytes, or what the request can make do with if that
+        exceeds the budget."""
+        return self.request_bytes(req)
+
     def launch(self, slot: int, reqs: Sequence[Request]):  # pragma: no cover - interface
         raise NotImplementedError
+
+    def launch_within(self, slot: int, reqs: Sequence[Request], nbytes: int):
+        """launch, holding no more than the bytes admitted for the group."""
+        return self.launch(slot, reqs)
 
     def done(self, handle) -> bool:  # pragma: no cover - interface
         raise NotImplementedError
@@ -164,7 +174,7 @@ class Scheduler:
             fut.set_exception(ValueError(f"unknown op {req.op!r}"))
             return fut
         try:
-            nbytes = self.ex.request_bytes(req)
+            nbytes = self.ex.fit_bytes(req, self.budget)
         except Exception as e:  # noqa: BLE001 - a request the executor cannot size is rejected
             fut.set_exception(e)
             return fut
@@ -281,7 +291,7 @@ class Scheduler:
                     self.in_use += nbytes
                     self.peak_in_use = max(self.peak_in_use, self.in_use)
                 try:
-                    handle = self.ex.launch(slot, [p.req for p in group])
+                    handle = self.ex.launch_within(slot, [p.req for p in group], nbytes)
                 except Exception as e:  # noqa: BLE001 - a failed launch rejects its group
                     with self._lock:
                         self.in_use -= nbytes
@@ -336,23 +346,33 @@ class GpuExecutor(Executor):
         with self._plock:
             self._pinned[(tuple(buf.shape), buf.dtype)].append(buf)
 
-    def request_bytes(self, req: Request) -> int:
-        """The request's buffers plus the library workspace its calls take
-        (the larger of the forward's and the back's for MBIR: they run one
-        after the other on one stream, whose pool reuses the memory)."""
-        from .binding import workspace_bytes
+    def _workspace(self, req: Request, limit: Optional[int] = None) -> int:
+        """Library workspace of a request's calls (the larger of the forward's
+        and the back's for MBIR: they run one after the other on one stream,
+        whose pool reuses the memory), the forward's within `limit`."""
+        from .binding import forward_workspace_within, workspace_bytes
         g = self.geometry(req.geometry)
         dt = self._dt[req.dtype]
+
+        def fwd():
+            return (workspace_bytes(g, req.projector, "fwd", dt) if limit is None else
+                    forward_workspace_within(g, req.projector, max(limit, 0), dt))
         if req.op == "fwd":
-            ws = workspace_bytes(g, req.projector, "fwd", dt)
-        elif req.op == "back":
-            ws = workspace_bytes(g, req.projector, "back", dt)
-        elif req.op == "mbir":
-            ws = max(workspace_bytes(g, req.projector, "fwd", dt),
-                     workspace_bytes(g, req.projector, "back", self.torch.float32))
-        else:
-            ws = workspace_bytes(g, "voxel", "back", self.torch.float32, mode="recon")
-        return request_bytes(req) + ws
+            return fwd()
+        if req.op == "back":
+            return workspace_bytes(g, req.projector, "back", dt)
+        if req.op == "mbir":
+            return max(fwd(), workspace_bytes(g, req.projector, "back", self.torch.float32))
+        return workspace_bytes(g, "voxel", "back", self.torch.float32, mode="recon")
+
+    def request_bytes(self, req: Request) -> int:
+        """The request's buffers plus the library workspace its calls take."""
+        return request_bytes(req) + self._workspace(req)
+
+    def fit_bytes(self, req: Request, budget: int) -> int:
+        own = request_bytes(req)
+        full = own + self._workspace(req)
+        return full if full <= budget else own + self._workspace(req, budget - own)
 
     def geometry(self, g: Dict[str, Any]):
         key = geometry_key(g)
@@ -369,6 +389,12 @@ class GpuExecutor(Executor):
         return self._lr[key]
 
     def launch(self, slot: int, reqs: Sequence[Request]):
+        return self._launch(slot, reqs, None)
+
+    def launch_within(self, slot: int, reqs: Sequence[Request], nbytes: int):
+        return self._launch(slot, reqs, max(0, nbytes - sum(request_bytes(r) for r in reqs)))
+
+    def _launch(self, slot: int, reqs: Sequence[Request], max_workspace: Optional[int]):
         from .binding import back_into, forward_into, ramp_filter
         from .mbir import ls_gradient_descent
         torch = self.torch
@@ -399,7 +425,7 @@ class GpuExecutor(Executor):
                 d_in = host_in.to(self.device, non_blocking=True)
             if r0.op == "fwd":
                 d_out = torch.empty((len(reqs),) + sino, dtype=dt, device=self.device)
-                forward_into(geom, d_in, d_out, r0.projector, stream=stream)
+                forward_into(geom, d_in, d_out, r0.projector, stream=stream, max_workspace=max_workspace)
             elif r0.op == "back":
                 d_out = torch.empty((len(reqs),) + vol, dtype=dt, device=self.device)
                 back_into(geom, d_in, d_out, r0.projector, stream=stream)
@@ -409,7 +435,8 @@ class GpuExecutor(Executor):
                 d_out = torch.empty((len(reqs),) + vol, dtype=dt, device=self.device)
                 back_into(geom, tmp, d_out, "voxel", mode="recon", stream=stream)
             else:
-                d_out = ls_gradient_descent(geom, d_in, r0.projector, r0.iters, lr=lr, stream=stream)
+                d_out = ls_gradient_descent(geom, d_in, r0.projector, r0.iters, lr=lr, stream=stream,
+                                            max_workspace=max_workspace)
             host_out = None
             if not r0.out_device:
                 host_out = self._pinned_buffer(tuple(d_out.shape), dt)

@@ -148,3 +148,28 @@ def test_admission_counts_the_library_workspace(ct):
     with pytest.raises(MemoryError):
         srv.submit(req).result(timeout=30)
     srv.close()
+
+
+@pytest.mark.parametrize("op,proj", [("fwd", "sf"), ("fwd", "ray"), ("mbir", "voxel")])
+def test_requests_that_fit_without_copies_are_admitted(ct, op, proj):
+    """A budget below a request's buffers and the copies of the volume that its forward likes to have: admitted, with
+    the same result, within the budget; refused only when the buffers do not fit."""
+    from paper_2503_16741_gb300.serve import Request, Server, request_bytes
+    sp = W.scaled(W.circ3d_256(), 64, 90)
+    data = np.random.default_rng(3).random(sp.vol_shape if op == "fwd" else sp.sino_shape).astype(np.float32)
+    req = Request(gdict(sp), op, data, projector=proj, iters=2)
+    srv = Server(device=0, slots=2, hbm_budget=1 << 30)
+    ref, ex = srv.submit(req).result(timeout=60), srv.ex
+    srv.close()
+    own, full = request_bytes(req), ex.request_bytes(req)
+    assert full > own
+    for budget in (full - 1, own):
+        srv = Server(hbm_budget=budget, executor=ex)
+        np.testing.assert_array_equal(srv.submit(req).result(timeout=60), ref)
+        assert srv.stats()["hbm_peak_bytes"] <= budget
+        srv.close()
+    srv = Server(hbm_budget=own - 1, executor=ex)
+    with pytest.raises(MemoryError):
+        srv.submit(req).result(timeout=30)
+    srv.close()
+    ct.workspace_limit(1 << 62)

@@ -75,6 +75,36 @@ def test_workspace_limit_releases_freed_blocks(ct):
     ct.workspace_limit(1 << 62)
 
 
+LIMITED = {"circ-flat": W.scaled(W.circ3d_256(), 64, 45), "circ-odd": W.scaled(W.circ3d_256(), 45, 40),
+           "circ-curved": W.scaled(W.circ3d_curved(), 64, 40) if hasattr(W, "circ3d_curved") else ragged("circ3d", "curved", 6),
+           "noncirc": ragged("noncirc3d", "flat", 8)}
+
+
+@pytest.mark.parametrize("name", LIMITED)
+@pytest.mark.parametrize("proj", ["voxel", "ray", "dd", "sf", "sftt"])
+def test_a_forward_without_its_copies_gives_the_same(ct, name, proj):
+    """Two copies of the volume, one, and none: the same projections bit for bit, and no more workspace than allowed."""
+    if proj == "sftt" and name == "circ-curved":
+        pytest.skip("SF-TT is for flat detectors")
+    g = ct.Geometry.from_spec(LIMITED[name])
+    x = torch.rand((2,) + g.vol_shape, device="cuda")
+    y = ct.forward(g, x, proj)
+    full = ct.workspace_bytes(g, proj, "fwd", batch=2)
+    for limit in (full, full - 1, full // 2, full // 2 - 1, 0):
+        if limit < 0:
+            continue
+        within = ct.forward_workspace_within(g, proj, limit, batch=2)
+        assert within <= limit
+        got = torch.empty_like(y)
+        torch.cuda.synchronize()
+        ct.workspace_usage(reset_high=True)
+        ct.forward_into(g, x, got, proj, max_workspace=limit)
+        torch.cuda.synchronize()
+        _, high = ct.workspace_usage()
+        assert high == 0 if within == 0 else within <= high <= within + GRANULE
+        assert torch.equal(got, y)
+
+
 def test_only_the_copies_that_the_views_need(ct):
     """Views whose central rays run along y, along x and along both."""
     spec = W.scaled(W.circ3d_256(), 64, 45)
