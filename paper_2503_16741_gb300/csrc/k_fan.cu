@@ -104,14 +104,13 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
     if (KIND == FAN_VOX) {
         float fu, rden2;
         fan_point<CURVED>(V, cu, cn, fu, rden2);
-        // a pixel that projects beside the detector reads none of its cells (one of
-        // them may be infinite or NaN, which a weight of zero would not hide)
-        if (fu <= -1.f || fu >= (float)g.nu) return;
         const float af = floorf(fu), t = fu - af;
         const int a0 = (int)af;
-        // at its ends, the cell off the detector weighs zero and reads the one on it
-        const float w0 = (unsigned)a0 < (unsigned)g.nu ? 1.f - t : 0.f;
-        const float w1 = (unsigned)(a0 + 1) < (unsigned)g.nu ? t : 0.f;
+        // at the detector's ends, the cell off it weighs zero and reads the one on it; a
+        // pixel that projects beside it adds nothing (an infinite or NaN cell times zero
+        // would be NaN; the last add is predicated, an early return cost 8 to 15 %)
+        const bool on0 = (unsigned)a0 < (unsigned)g.nu, on1 = (unsigned)(a0 + 1) < (unsigned)g.nu;
+        const float w0 = on0 ? 1.f - t : 0.f, w1 = on1 ? t : 0.f;
         float amp = V.rc_w * rden2;
         if (!RECON) {
             const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
@@ -120,8 +119,10 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
         }
         const int c0 = min(max(a0, 0), g.nu - 1), c1 = min(max(a0 + 1, 0), g.nu - 1);
 #pragma unroll
-        for (int q = 0; q < NBT; ++q, y += ystride)
-            acc[q] = fmaf(amp, fmaf(w1, ld(y, (size_t)c1), w0 * ld(y, (size_t)c0)), acc[q]);
+        for (int q = 0; q < NBT; ++q, y += ystride) {
+            const float s = fmaf(w1, ld(y, (size_t)c1), w0 * ld(y, (size_t)c0));
+            if (on0 || on1) acc[q] = fmaf(amp, s, acc[q]);
+        }
     } else if (KIND == FAN_RAY) {
         int aref;
         float k[4];
