@@ -505,7 +505,7 @@ static size_t workspace_rule(int dir, const ct_geometry *g, ct_projector proj, c
     if (dir == 0) {
         switch (proj) {
         case CT_VOXEL: return ctp::circ_fwd_fits(G, ctp::BK_VOX, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;
-        case CT_RAY: return G.is2d || !G.ray_x ? 0 : vox * isz;
+        case CT_RAY: return G.is2d || !ctp::ray_copies(G, batch) ? 0 : vox * isz;
         case CT_DD:
             if (nc) return ctp::nc_footprint_fits(G, 1) ? vox * isz : 0;
             return ctp::circ_fwd_fits(G, ctp::BK_DD, batch) ? ctp::circ_fwd_workspace(G, batch, (int)isz) : 0;

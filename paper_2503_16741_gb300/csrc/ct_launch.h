@@ -93,8 +93,14 @@ cudaError_t zmajor_copy(int elem_bytes, const void *x, void *xZ, int nx, int ny,
 inline int zmajor_pitch(const CtGrid &g) {
     return g.is2d || g.variant == GEO_NONCIRC_FLAT || g.nz < 4 ? 0 : (g.nz + 3) & ~3;
 }
+// Volumes of at most this many voxels (32^3) go without reordered copies, which would
+// cost the smallest calls an allocation and a launch
+constexpr long long kCopyVoxels = 32768;
+inline bool copies_pay(const CtGrid &g, int batch) { return (long long)g.nx * g.ny * g.nz * batch > kCopyVoxels; }
+// the ray-driven forward's copy
+inline bool ray_copies(const CtGrid &g, int batch) { return g.ray_x && copies_pay(g, batch); }
 // the copy's grid (rows and batch items are its y and z)
-inline bool zmajor_copy_fits(const CtGrid &g, int batch) { return batch <= 65535 && g.ny <= 65535; }
+inline bool zmajor_copy_fits(const CtGrid &g, int batch) { return copies_pay(g, batch) && batch <= 65535 && g.ny <= 65535; }
 
 // Stream-ordered scratch from a library-owned pool on the current device
 // (memory is kept in the pool between calls, so steady-state calls do not

@@ -53,10 +53,10 @@ struct FwdVolume {
     const void *y, *x;
     int nzp;
 };
-// Volumes of at most 32^3 voxels in calls of few CTAs are read in place: the copies
-// would cost such a call an allocation and a launch, a third of its time.
+// The smallest volumes are read in place in calls of few CTAs: the copies would cost
+// such a call an allocation and a launch, a third of its time.
 inline bool circ_fwd_direct(const CtGrid &g, int batch) {
-    return (long long)g.nx * g.ny * g.nz * batch <= 32768 && circ_fwd_ctas(g, 32, batch) < kFwdWave;
+    return !copies_pay(g, batch) && circ_fwd_ctas(g, 32, batch) < kFwdWave;
 }
 
 namespace {

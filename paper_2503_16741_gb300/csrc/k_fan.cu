@@ -343,7 +343,7 @@ fan_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
     st_out(g, sino, ((size_t)(bt + w) * g.nview + v) * g.nu + a, s * fan_cell_factor<KIND, CURVED>(V, g, a), out_t);
 }
 
-// Ray-driven forward: thread = (ray, one of 8 runs of slabs), see ray_run.
+// Ray-driven forward: thread = (ray, one of 8 runs of slabs), see ray_runs.
 template <typename TIn, bool CURVED>
 __global__ void __launch_bounds__(32 * kFanWarps)
 fan_ray_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, void *__restrict__ sino,
@@ -355,10 +355,10 @@ fan_ray_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ 
     const int v = bx % g.nview;
     const int bt = bx / g.nview;
     const int a = tu * 32 + lane;
-    float acc = 0.f, len = 0.f;
+    float acc[1] = {0.f}, len = 0.f;
     if (a < g.nu)
-        acc = ray_run<TIn, CURVED, true, kFanWarps>(views[v], g, a, 0, vol + (size_t)bt * g.nx * g.ny, nullptr, w, len);
-    red[w][lane] = acc;
+        ray_runs<TIn, CURVED, true, kFanWarps, 1>(views[v], g, a, 0, vol + (size_t)bt * g.nx * g.ny, nullptr, w, len, acc);
+    red[w][lane] = acc[0];
     __syncthreads();
     if (w || a >= g.nu) return;
     float s = red[0][lane];

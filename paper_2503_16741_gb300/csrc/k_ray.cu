@@ -19,10 +19,14 @@
 namespace ctp {
 
 // ------------------------------------------------------------ forward
-// Thread = (ray, one of kRayGroups runs of slabs): 32 x 2 rays, whose runs are
-// added through shared memory in a fixed order.  Bound by instruction issue (79 %
-// of slots).  128^3 / 180 views / 256 x 192: 1.66 ms with a merged-crossing walk
-// per ray, 1.13 ms so (with the copy that rays along x read).
+// A ray's kRayGroups runs of slabs are summed by a thread each (TPR = 4), whose sums
+// are added through shared memory, or by one thread, which sets the ray up once
+// (TPR = 1), in the same order: the choice changes no bit, so it may follow the number
+// of rays.  One thread for volumes of up to 64 slabs, whose rays are not much longer
+// than their set-up, from 1.5 waves of rays on: curved 54 x 22 x 54 / 359 views / 158 x
+// 72, three volumes, 4 threads 1.24 ms, 1 thread 0.82; 64^3 / 180 views / 128 x 96 374,
+// 312 us.  128^3 / 180 views / 256 x 192 2.14 ms (3.73 with a merged-crossing walk per
+// ray).  Bound by instruction issue.
 constexpr int kRayGroups = 4;
 
 // xT[k][i][j] = x[k][j][i] of every slice: rays along x step through the copy
@@ -45,30 +49,38 @@ swap_xy(const T *__restrict__ x, T *__restrict__ xT, int nx, int ny, long long s
     }
 }
 
-template <typename TIn, bool CURVED>
+template <typename TIn, bool CURVED, int TPR>
 __global__ void __launch_bounds__(256)
 ray_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, const TIn *__restrict__ volT,
         void *__restrict__ sino, int out_t, int tiles_u) {
-    __shared__ float red[kRayGroups][64];
+    static_assert(TPR == 1 || TPR == kRayGroups, "all runs or one to a thread");
+    constexpr int RY = 8 / TPR, N = kRayGroups / TPR;  // rows of rays of the block, runs of a thread
+    __shared__ float red[TPR][32 * RY];
     int bx = blockIdx.x;
     const int tu = bx % tiles_u; bx /= tiles_u;
     const int v = bx % g.nview;
     const int bt = bx / g.nview;
-    // 32 x 2 rays x kRayGroups runs of slabs
-    const int ry = threadIdx.y & 1, grp = threadIdx.y >> 1, slot = ry * 32 + threadIdx.x;
+    const int ry = threadIdx.y % RY, grp = threadIdx.y / RY, slot = ry * 32 + threadIdx.x;
     const int a = tu * 32 + threadIdx.x;
-    const int b = blockIdx.y * 2 + ry;
+    const int b = blockIdx.y * RY + ry;
     const size_t nvox = (size_t)g.nx * g.ny * g.nz;
-    float acc = 0.f, len = 0.f;
+    float sum[N] = {}, len = 0.f;
     if (a < g.nu && b < g.nv)
-        acc = ray_run<TIn, CURVED, false, kRayGroups>(views[v], g, a, b, vol + bt * nvox, volT ? volT + bt * nvox : nullptr,
-                                               grp, len);
-    red[grp][slot] = acc;
-    __syncthreads();
-    if (grp || a >= g.nu || b >= g.nv) return;
-    float s = red[0][slot];
+        ray_runs<TIn, CURVED, false, kRayGroups, N>(views[v], g, a, b, vol + bt * nvox, volT ? volT + bt * nvox : nullptr,
+                                                    grp * N, len, sum);
+    float s = sum[0];
+    if (TPR > 1) {
+        red[grp][slot] = s;
+        __syncthreads();
+        if (grp) return;
+        s = red[0][slot];
 #pragma unroll
-    for (int q = 1; q < kRayGroups; ++q) s += red[q][slot];
+        for (int q = 1; q < TPR; ++q) s += red[q][slot];
+    } else {
+#pragma unroll
+        for (int q = 1; q < N; ++q) s += sum[q];
+    }
+    if (a >= g.nu || b >= g.nv) return;
     st_out(g, sino, (((size_t)bt * g.nview + v) * g.nv + b) * g.nu + a, s * len, out_t);
 }
 
@@ -414,7 +426,7 @@ cudaError_t ray_launch_t(int dir, const CtGrid &g, const CtView *views, const vo
         const int tiles_u = (g.nu + 31) / 32;
         TIn *xT = nullptr;  // for rays along x, where there may be some (without it they read strided)
         const long long slices = (long long)g.nz * batch;
-        if (!g.ray_x) {
+        if (!ray_copies(g, batch)) {
         } else if (workspace_alloc_copy((void **)&xT, (size_t)g.nx * g.ny * slices * sizeof(TIn), g, st) != cudaSuccess) {
             cudaGetLastError();
             xT = nullptr;
@@ -422,11 +434,13 @@ cudaError_t ray_launch_t(int dir, const CtGrid &g, const CtView *views, const vo
             const dim3 tg((unsigned)(((g.nx + 31) / 32) * ((g.ny + 31) / 32)), (unsigned)std::min(slices, 65535LL));
             swap_xy<TIn><<<tg, dim3(32, 8), 0, st>>>(src, xT, g.nx, g.ny, slices);
         }
-        dim3 blk(32, 2 * kRayGroups), grd((unsigned)(tiles_u * g.nview * batch), (unsigned)((g.nv + 1) / 2));
-        if (g.variant == GEO_CIRC_CURVED)
-            ray_fwd<TIn, true><<<grd, blk, 0, st>>>(g, views, src, xT, out, out_t, tiles_u);
-        else
-            ray_fwd<TIn, false><<<grd, blk, 0, st>>>(g, views, src, xT, out, out_t, tiles_u);
+        const bool one = std::max(std::max(g.nx, g.ny), g.nz) <= 64 && (long long)g.nu * g.nv * g.nview * batch >= 3 * 152 * 1024LL;
+        const int rows = one ? 8 : 8 / kRayGroups;
+        dim3 blk(32, 8), grd((unsigned)(tiles_u * g.nview * batch), (unsigned)((g.nv + rows - 1) / rows));
+        const bool curved = g.variant == GEO_CIRC_CURVED;
+        auto kern = one ? (curved ? ray_fwd<TIn, true, 1> : ray_fwd<TIn, false, 1>)
+                        : (curved ? ray_fwd<TIn, true, kRayGroups> : ray_fwd<TIn, false, kRayGroups>);
+        kern<<<grd, blk, 0, st>>>(g, views, src, xT, out, out_t, tiles_u);
         const cudaError_t e = cudaGetLastError();
         const cudaError_t ef = workspace_free(xT, st);
         return e != cudaSuccess ? e : ef;

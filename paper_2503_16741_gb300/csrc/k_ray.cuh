@@ -23,8 +23,9 @@ __device__ __forceinline__ void ray_dir(const CtView &V, const CtGrid &g, int a,
     for (int m = 0; m < 3; ++m) d[m] = fmaf(cn_, V.nn[m], fmaf(cu_, V.eu[m], Vb * V.ev[m]));
 }
 
-// Sum of chord x value over the grp-th of NG runs of slabs of the ray of cell
-// (a, b); the caller adds the runs and multiplies by the ray's length `len`.
+// Sums of chord x value over the runs grp, grp + 1, .. (N of them) of NG runs of slabs
+// of the ray of cell (a, b); the caller adds the runs and multiplies by the ray's
+// length `len`.  (A run's sum is the same whichever thread forms it.)
 // TWO: fan beam, the ray stays in the one slice.
 //
 // The chord lengths are Siddon's, taken slab by slab along the axis on which the
@@ -36,9 +37,9 @@ __device__ __forceinline__ void ray_dir(const CtView &V, const CtGrid &g, int a,
 // the same slab, so their loads coalesce.  Axes along which the ray descends are
 // mirrored (indices and strides negated).  volT (may be null): a copy of the
 // volume whose fastest axis is y, for rays along x.
-template <typename TIn, bool CURVED, bool TWO, int NG>
-__device__ __forceinline__ float ray_run(const CtView &V, const CtGrid &g, int a, int b, const TIn *__restrict__ vol,
-                                         const TIn *__restrict__ volT, int grp, float &len) {
+template <typename TIn, bool CURVED, bool TWO, int NG, int N>
+__device__ __forceinline__ void ray_runs(const CtView &V, const CtGrid &g, int a, int b, const TIn *__restrict__ vol,
+                                         const TIn *__restrict__ volT, int grp, float &len, float (&sum)[N]) {
     constexpr int NAX = TWO ? 2 : 3;
     float d[3];
     ray_dir<CURVED>(V, g, a, b, d);
@@ -61,7 +62,9 @@ __device__ __forceinline__ float ray_run(const CtView &V, const CtGrid &g, int a
             tout = fminf(tout, fmaxf(t1, t2));
         }
     }
-    if (!(hit && tout > tin)) return 0.f;
+#pragma unroll
+    for (int q = 0; q < N; ++q) sum[q] = 0.f;
+    if (!(hit && tout > tin)) return;
     const float T = tout - tin;
     // mirrored axes: entry point, speed, crossing-parameter step, index range
     float q[3], inv[3], lo[3], hi[3];
@@ -95,56 +98,61 @@ __device__ __forceinline__ float ray_run(const CtView &V, const CtGrid &g, int a
     const float c0 = index(qm, pick(lo, 0), um);  // entry slab
     // slabs to the volume's end, or to the ray's
     const int nsl = (int)fminf(um - c0 + 1.f, floorf(T * Dm) + 3.f), per = (nsl + NG - 1) / NG;
-    const int i0 = grp * per, i1 = min(i0 + per, nsl);
-    if (i0 >= i1) return 0.f;
-    float cm = c0 + (float)i0;  // the slab's index
-    float ta = i0 == 0 ? 0.f : fminf(fmaxf((cm - 0.5f - qm) * im, 0.f), T);
     constexpr float kNever = 3.0e38f;
-    // lateral index, and the parameter at which the next one begins
-    const float qp = pick(q, 1), ip = pick(inv, 1), up = pick(hi, 1);
-    float jp = index(fmaf(ta, pick(D, 1), qp), pick(lo, 1), up);
-    float np = ip != 0.f && jp < up ? (jp + 0.5f - qp) * ip : kNever;
-    ptrdiff_t off = (ptrdiff_t)cm * tm + (ptrdiff_t)jp * tp;
-    float qr = 0.f, ir = 0.f, ur = 0.f, jr = 0.f, nr = kNever;
-    if (!TWO) {
-        qr = pick(q, 2); ir = pick(inv, 2); ur = pick(hi, 2);
-        jr = index(fmaf(ta, pick(D, 2), qr), pick(lo, 2), ur);
-        nr = ir != 0.f && jr < ur ? (jr + 0.5f - qr) * ir : kNever;
-        off += (ptrdiff_t)jr * tr;
-    }
-    const TIn *x = (swap ? volT : vol) + off;
-    float acc = 0.f;
-    for (int i = i0; i < i1 && ta < T; ++i, x += tm, cm += 1.f) {
-        const float te = fminf(fmaxf((cm + 0.5f - qm) * im, ta), T);
-        const bool xp = np < te, xr = !TWO && nr < te;
-        const float cp = xp ? fmaxf(np, ta) : te, cr = xr ? fmaxf(nr, ta) : te;
-        const float e1 = TWO ? cp : fminf(cp, cr);
-        acc = fmaf(e1 - ta, ld(x, 0), acc);
-        if (TWO) {
-            if (xp) {
-                x += tp;
-                acc = fmaf(te - cp, ld(x, 0), acc);
-                jp += 1.f;
-                np = jp < up ? (jp + 0.5f - qp) * ip : kNever;
-            }
-        } else if (xp || xr) {
-            const float e2 = fmaxf(cp, cr);
-            acc = fmaf(e2 - e1, ld(x + (xp && (!xr || cp < cr) ? tp : tr), 0), acc);
-            if (xp) {
-                x += tp;
-                jp += 1.f;
-                np = jp < up ? (jp + 0.5f - qp) * ip : kNever;
-            }
-            if (xr) {
-                x += tr;
-                jr += 1.f;
-                nr = jr < ur ? (jr + 0.5f - qr) * ir : kNever;
-            }
-            if (xp && xr) acc = fmaf(te - e2, ld(x, 0), acc);
+#pragma unroll 1
+    for (int run = 0; run < N; ++run) {
+        const int i0 = (grp + run) * per, i1 = min(i0 + per, nsl);
+        if (i0 >= i1) return;
+        float cm = c0 + (float)i0;  // the slab's index
+        float ta = i0 == 0 ? 0.f : fminf(fmaxf((cm - 0.5f - qm) * im, 0.f), T);
+        // lateral index, and the parameter at which the next one begins
+        const float qp = pick(q, 1), ip = pick(inv, 1), up = pick(hi, 1);
+        float jp = index(fmaf(ta, pick(D, 1), qp), pick(lo, 1), up);
+        float np = ip != 0.f && jp < up ? (jp + 0.5f - qp) * ip : kNever;
+        ptrdiff_t off = (ptrdiff_t)cm * tm + (ptrdiff_t)jp * tp;
+        float qr = 0.f, ir = 0.f, ur = 0.f, jr = 0.f, nr = kNever;
+        if (!TWO) {
+            qr = pick(q, 2); ir = pick(inv, 2); ur = pick(hi, 2);
+            jr = index(fmaf(ta, pick(D, 2), qr), pick(lo, 2), ur);
+            nr = ir != 0.f && jr < ur ? (jr + 0.5f - qr) * ir : kNever;
+            off += (ptrdiff_t)jr * tr;
         }
-        ta = te;
+        const TIn *x = (swap ? volT : vol) + off;
+        float acc = 0.f;
+        for (int i = i0; i < i1 && ta < T; ++i, x += tm, cm += 1.f) {
+            const float te = fminf(fmaxf((cm + 0.5f - qm) * im, ta), T);
+            const bool xp = np < te, xr = !TWO && nr < te;
+            const float cp = xp ? fmaxf(np, ta) : te, cr = xr ? fmaxf(nr, ta) : te;
+            const float e1 = TWO ? cp : fminf(cp, cr);
+            acc = fmaf(e1 - ta, ld(x, 0), acc);
+            if (TWO) {
+                if (xp) {
+                    x += tp;
+                    acc = fmaf(te - cp, ld(x, 0), acc);
+                    jp += 1.f;
+                    np = jp < up ? (jp + 0.5f - qp) * ip : kNever;
+                }
+            } else if (xp || xr) {
+                const float e2 = fmaxf(cp, cr);
+                acc = fmaf(e2 - e1, ld(x + (xp && (!xr || cp < cr) ? tp : tr), 0), acc);
+                if (xp) {
+                    x += tp;
+                    jp += 1.f;
+                    np = jp < up ? (jp + 0.5f - qp) * ip : kNever;
+                }
+                if (xr) {
+                    x += tr;
+                    jr += 1.f;
+                    nr = jr < ur ? (jr + 0.5f - qr) * ir : kNever;
+                }
+                if (xp && xr) acc = fmaf(te - e2, ld(x, 0), acc);
+            }
+            ta = te;
+        }
+        // (registers, for any N)
+#pragma unroll
+        for (int q = 0; q < N; ++q) sum[q] = q == run ? acc : sum[q];
     }
-    return acc;
 }
 
 }  // namespace ctp

@@ -224,3 +224,16 @@ def test_a_view_does_not_depend_on_the_others(ct, proj, du, dv):
     _check(y.cpu().numpy(), oracle.forward(spec, proj, x.double().cpu().numpy()), "forward")
     for views in (list(range(0, nview, 2)), list(range(1, nview, 2)), [4]):
         assert torch.equal(ct.forward(g.subset(views), x, proj), y[views])
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+def test_ray_forward_by_one_thread_or_four(ct, det):
+    """A ray's runs of slabs, each by a thread of its own in small calls and all by one in large ones, add up alike."""
+    spec = _spec(det, 41, 23, 60, 150, 150, 24, 1.0, 1.1)
+    assert spec.nu * spec.nv * spec.nview >= 3 * 152 * 1024 > spec.nu * spec.nv * 8
+    g = ct.Geometry.from_spec(spec)
+    x = torch.as_tensor(W.random_volume(spec, seed=2)[0] - 0.3, dtype=torch.float32).cuda()
+    y = ct.forward(g, x, "ray")
+    _check(y.cpu().numpy(), oracle.forward(spec, "ray", x.double().cpu().numpy()), "forward")
+    for views in (list(range(0, 24, 3)), [5], [23]):
+        assert torch.equal(ct.forward(g.subset(views), x, "ray"), y[views])
