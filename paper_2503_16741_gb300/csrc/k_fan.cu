@@ -94,8 +94,10 @@ __device__ __forceinline__ void fan_slab(float w, float e, float h, float &lo, f
 
 // ------------------------------------------------------------ back (gather)
 // adds one view's contributions to pixel (i, j) of NBT batch items, whose rows
-// y are ystride apart (the footprint is formed once for all of them)
-template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT>
+// y are ystride apart (the footprint is formed once for all of them).  OWN
+// (voxel-driven): a pixel that projects beside the detector adds nothing, rather than
+// its end cell with a weight of zero.
+template <typename TIn, int KIND, bool CURVED, bool RECON, int NBT, bool OWN = false>
 __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, const TIn *__restrict__ y,
                                               size_t ystride, int i, int j, float (&acc)[NBT]) {
     const float fi = (float)i, fj = (float)j;
@@ -106,11 +108,10 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
         fan_point<CURVED>(V, cu, cn, fu, rden2);
         const float af = floorf(fu), t = fu - af;
         const int a0 = (int)af;
-        // at the detector's ends, the cell off it weighs zero and reads the one on it; a
-        // pixel that projects beside it adds nothing (an infinite or NaN cell times zero
-        // would be NaN; the last add is predicated, an early return cost 8 to 15 %)
-        const bool on0 = (unsigned)a0 < (unsigned)g.nu, on1 = (unsigned)(a0 + 1) < (unsigned)g.nu;
-        const float w0 = on0 ? 1.f - t : 0.f, w1 = on1 ? t : 0.f;
+        if (OWN && (fu <= -1.f || fu >= (float)g.nu)) return;
+        // cells off the detector weigh zero and read a clamped address
+        const float w0 = (unsigned)a0 < (unsigned)g.nu ? 1.f - t : 0.f;
+        const float w1 = (unsigned)(a0 + 1) < (unsigned)g.nu ? t : 0.f;
         float amp = V.rc_w * rden2;
         if (!RECON) {
             const float wx = fmaf(fi, g.dx, V.o[0]), wy = fmaf(fj, g.dy, V.o[1]);
@@ -119,10 +120,8 @@ __device__ __forceinline__ void fan_back_view(const CtView &V, const CtGrid &g, 
         }
         const int c0 = min(max(a0, 0), g.nu - 1), c1 = min(max(a0 + 1, 0), g.nu - 1);
 #pragma unroll
-        for (int q = 0; q < NBT; ++q, y += ystride) {
-            const float s = fmaf(w1, ld(y, (size_t)c1), w0 * ld(y, (size_t)c0));
-            if (on0 || on1) acc[q] = fmaf(amp, s, acc[q]);
-        }
+        for (int q = 0; q < NBT; ++q, y += ystride)
+            acc[q] = fmaf(amp, fmaf(w1, ld(y, (size_t)c1), w0 * ld(y, (size_t)c0)), acc[q]);
     } else if (KIND == FAN_RAY) {
         int aref;
         float k[4];
@@ -223,6 +222,24 @@ fan_back(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ sin
                         if (e == 0 || j + 4 * e < g.ny)
                             fan_back_view<TIn, KIND, CURVED, RECON, NBT>(sview[t], g, ys + (size_t)(v0 + t) * g.nu,
                                                                          ystride, i, j + 4 * e, acc[e]);
+        }
+        if constexpr (KIND == FAN_VOX) {
+            // An infinite or NaN cell at an end of the detector makes the sums of the pixels
+            // beyond it NaN (zero times it): a thread with such a sum starts again without
+            // them.  (A test per view cost the kernel 2 to 15 %.)
+            float bad = 0.f;
+#pragma unroll
+            for (int q = 0; q < PX * NBT; ++q) bad = fmaf(acc[q / NBT][q % NBT], 0.f, bad);
+            if (bad != 0.f) {
+#pragma unroll
+                for (int q = 0; q < PX * NBT; ++q) acc[q / NBT][q % NBT] = 0.f;
+                for (int v = w; v < g.nview; v += kFanWarps)
+#pragma unroll
+                    for (int e = 0; e < PX; ++e)
+                        if (e == 0 || j + 4 * e < g.ny)
+                            fan_back_view<TIn, KIND, CURVED, RECON, NBT, true>(views[v], g, ys + (size_t)v * g.nu, ystride, i,
+                                                                               j + 4 * e, acc[e]);
+            }
         }
 #pragma unroll
         for (int q = 0; q < PX * NBT; ++q) red[q][w][lane] = acc[q / NBT][q % NBT];
