@@ -90,3 +90,37 @@ def test_a_bad_edge_cell_stays_on_the_detector(ct, det, mode, size):
     touched = oracle.back(spec, "voxel", mask).reshape(g.vol_shape) != 0
     assert not ok.all() and torch.equal(bad[ok], clean[ok])
     assert not (~ok.cpu().numpy() & ~touched).any()
+
+
+@pytest.mark.parametrize("det", ["flat", "curved"])
+@pytest.mark.parametrize("proj,mode", [("voxel", "proj"), ("voxel", "recon"), ("sf", "proj"), ("dd", "recon"), ("ray", "proj")])
+def test_two_pixels_to_a_thread(ct, det, proj, mode):
+    """Images of 65536 pixels and more, alone: patches of 8 x 8 with remainders of 3 columns and of 5 and 1 rows. The
+    same image in a pair takes one pixel to a thread: equal bit for bit; footprints besides against the oracle (the
+    other two read positions along the whole detector, whose rounding exceeds this bound at 300 cells)."""
+    for nx, ny in ((259, 261), (259, 257)):
+        assert nx * ny >= 65536
+        spec = _spec(det, nx, ny, 300, 11, 259 * 1.6 * 2 * 0.9 / 300)
+        g = ct.Geometry.from_spec(spec)
+        q = W.random_sino(spec, seed=3)[0]
+        y = torch.as_tensor(q[:, 0], dtype=torch.float32).cuda()
+        got = ct.back(g, y, proj, mode=mode)
+        assert torch.equal(got, ct.back(g, torch.stack([y, 1 - y]), proj, mode=mode)[0])
+        if proj in ("sf", "dd"):
+            ref = oracle.back(spec, proj, q) if mode == "proj" else oracle.back_recon(spec, q, proj)
+            _same(got.cpu().numpy(), ref.reshape(g.vol_shape), proj)
+
+
+@pytest.mark.parametrize("batch", [3, 5])
+@pytest.mark.parametrize("tin,tout", [("f32", "f32"), ("f16", "f16"), ("f32", "bf16"), ("bf16", "f32")])
+@pytest.mark.parametrize("proj", ["sf", "dd", "voxel", "ray"])
+def test_the_item_after_the_pairs(ct, proj, tin, tout, batch):
+    """Odd batches: pairs and one item alone, at its own offset for every storage type, each as by itself."""
+    T = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}
+    g = ct.Geometry.from_spec(_spec("flat", 31, 45, 77, 9, 1.5))
+    x = torch.rand((batch,) + g.vol_shape, device="cuda").to(T[tin])
+    y = torch.rand((batch,) + g.sino_shape, device="cuda").to(T[tin])
+    Ax, Aty = ct.forward(g, x, proj, out_dtype=T[tout]), ct.back(g, y, proj, out_dtype=T[tout])
+    for b in range(batch):
+        assert torch.equal(Ax[b], ct.forward(g, x[b].contiguous(), proj, out_dtype=T[tout]))
+        assert torch.equal(Aty[b], ct.back(g, y[b].contiguous(), proj, out_dtype=T[tout]))
