@@ -193,7 +193,7 @@ def serving_mix(n_req: int, seed: int = 0):
     40 % / back 40 % / 10-step least-squares MBIR 20 %, SF or DD.  Bounded so
     that 500 requests run in tens of seconds: MBIR volumes at most 256^3
     (non-circular 128^3), non-circular volumes at most 256^3 (the
-    non-circular kernels take about ten times longer per update).
+    non-circular kernels take about eight times longer per update).
     Returns [(request fields, voxel-view updates)]."""
     import numpy as np
 

@@ -1,7 +1,7 @@
 // ct_workspace.cpp -- stream-ordered scratch memory for kernels that need a
 // buffer beyond their inputs and outputs (the scaled FP32 sinograms of the
-// DD, SF-TT and circular ray-driven backs, the z-major volume copy of the
-// footprint and voxel-driven forwards).  One memory pool per device, created
+// DD, SF-TT and circular ray-driven backs, the reordered copies of the volume of
+// the forwards, which can do without them).  One memory pool per device, created
 // on first use, whose release threshold keeps freed blocks for reuse (all of
 // them by default; ct_workspace_limit caps what is kept).
 #include <cuda_runtime.h>

@@ -25,7 +25,7 @@
 // The split depends on the geometry alone: deterministic, and batch items do
 // not depend on the batch.
 //
-// Bound by instruction issue (69 % of slots) and L1 (52 %), the row loads first.
+// Bound by instruction issue, then L1: the row loads first.
 // Measured against the kernels before (set-up per chunk, four taps for every
 // footprint, a step-by-step sweep; one column walk per block of views for tall
 // voxels), 256^3 / 360 views / 512 x 384 FP32: SF-TR 10.63 -> 7.23 ms, voxel-

@@ -12,14 +12,13 @@
 //            items that reach its cell and adds weight x axial projection.
 // Each sum has a fixed order: deterministic, and no atomics.  The walk reads a
 // copy of the volume in groups of four voxels down z, [z/4][slab][lateral][4],
-// one for either main axis: a warp's load is 32 adjacent columns (512
+// one for each main axis that the views have: a warp's load is 32 adjacent columns (512
 // contiguous bytes of FP32; in a column-contiguous copy every lane touched a
 // cache line of its own, a quarter of the L1 traffic).  The copy pads z with
 // zeros, so every height takes the same walk (heights that are no multiple of
 // four used to be read voxel by voxel across the slices).
 //
-// Both stages are bound by instruction issue (66 % of slots) and the L1/shared
-// pipe (55 %).  The walk runs in packed FP32x2: the position of a voxel's edge
+// Both stages are bound by instruction issue and the L1/shared pipe.  The walk runs in packed FP32x2: the position of a voxel's edge
 // is formed from its index alone (no chain from voxel to voxel), rounded to its
 // row by adding 1.5 2^23, whose low bits then are the row's offset in shared
 // memory; a closed row is stored by one predicated instruction (as a branch it
@@ -29,7 +28,7 @@
 // Of the 256^3 scan's time (11.4 ms before the 64-cell tiles), compiling parts
 // out left: set-up and search 1.3 ms, walk 5.6, stage 2 5.0.
 // Measured against the kernel before, 256^3 / 360 views / 512 x 384 FP32: SF-TR
-// 13.4 -> 10.7 ms, voxel-driven 19.2 -> 10.4 ms; 161^2 x 155 / 607 views, SF-TR
+// 13.4 -> 10.6 ms, voxel-driven 19.2 -> 10.2 ms; 161^2 x 155 / 607 views, SF-TR
 // 10.4 -> 5.1 ms (no multiple of four slices); 183^2 x 157 / 231 views, DD with
 // voxels up to 1.2 rows high 6.4 -> 3.7 ms; curved 512^2 x 128 / 984 views, DD
 // 65.3 -> 48 ms.

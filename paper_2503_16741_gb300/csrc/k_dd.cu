@@ -1,12 +1,12 @@
 // k_dd.cu -- distance-driven projector (De Man & Basu 2004, cited in Sec.
-// 2.3) in non-circular geometry (the circular kernels share the footprint
-// kernels of k_sf.cu).  Per view the slabs run along the main axis (x or y, whichever the
-// central ray follows more closely).  A voxel's transaxial boundary points
-// (+- half a voxel along the other axis) and axial boundary points
-// (+- dz/2) are projected to the detector; the weight of cell (a, b) is
-// (u overlap / du) (v overlap / dv) L_c, with L_c = slab width / |d_main| the
-// path of the cell's central ray through one slab.  Gather kernels for both
-// directions, sharing the weight functions.
+// 2.3) in non-circular geometry, for footprints beyond those of k_nc.cuh (the
+// circular kernels are those of k_circ_fwd.cuh and k_circ_back.cuh).  Per view
+// the slabs run along the main axis (x or y, whichever the central ray follows
+// more closely).  A voxel's transaxial boundary points (+- half a voxel along
+// the other axis) and axial boundary points (+- dz/2) are projected to the
+// detector; the weight of cell (a, b) is (u overlap / du) (v overlap / dv) L_c,
+// with L_c = slab width / |d_main| the path of the cell's central ray through
+// one slab.  Gather kernels for both directions, sharing the weight functions.
 #include "ct_device.cuh"
 #include "ct_launch.h"
 

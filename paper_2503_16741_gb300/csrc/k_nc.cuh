@@ -158,28 +158,22 @@ __device__ __forceinline__ void nc_fp(const CtView &V, const CtGrid &g, const Nc
     P.a0 = aref + d0;
     const float hzv = V.hzv, hzn = V.hzn;
     if (KIND == NC_TT) {
-        if (g.is2d) {  // one row of unit height, inside the axial plateau: factor 1
-#pragma unroll
-            for (int q = 0; q < NB; ++q) P.Fv[q] = q == 0 ? 1.f : 0.f;
-            P.b0 = 0;
-        } else {
-            const float eps = 1e-7f * g.dx;
-            const float hxn = 0.5f * V.an[0], hyn = 0.5f * V.an[1];
-            const float hxv = 0.5f * V.av[0], hyv = 0.5f * V.av[1];
-            const float snx = V.an[0] < -eps ? 1.f : -1.f, sny = V.an[1] < -eps ? 1.f : -1.f;  // nearest
-            const float sfx = V.an[0] > eps ? 1.f : -1.f, sfy = V.an[1] > eps ? 1.f : -1.f;    // farthest
-            const float nv_ = fmaf(snx, hxv, sny * hyv), nn_ = fmaf(snx, hxn, sny * hyn);
-            const float fv_ = fmaf(sfx, hxv, sfy * hyv), fn_ = fmaf(sfx, hxn, sfy * hyn);
-            float t0 = vr + V.Kv * __fdividef(fmaf(-rv, nn_ - hzn, nv_ - hzv), cn + nn_ - hzn);
-            float t1 = vr + V.Kv * __fdividef(fmaf(-rv, nn_ + hzn, nv_ + hzv), cn + nn_ + hzn);
-            float t2 = vr + V.Kv * __fdividef(fmaf(-rv, fn_ - hzn, fv_ - hzv), cn + fn_ - hzn);
-            float t3 = vr + V.Kv * __fdividef(fmaf(-rv, fn_ + hzn, fv_ + hzv), cn + fn_ + hzn);
-            sort4(t0, t1, t2, t3);
-            const Trap Tv = nc_trap(t0, t1, t2, t3);
-            const int e0 = (int)floorf(Tv.k0 + 0.5f), e1 = (int)floorf(Tv.k3 + 0.5f);
-            nc_cells<NB>(Tv, e0, e1, P.Fv);
-            P.b0 = bref + e0;
-        }
+        const float eps = 1e-7f * g.dx;
+        const float hxn = 0.5f * V.an[0], hyn = 0.5f * V.an[1];
+        const float hxv = 0.5f * V.av[0], hyv = 0.5f * V.av[1];
+        const float snx = V.an[0] < -eps ? 1.f : -1.f, sny = V.an[1] < -eps ? 1.f : -1.f;  // nearest
+        const float sfx = V.an[0] > eps ? 1.f : -1.f, sfy = V.an[1] > eps ? 1.f : -1.f;    // farthest
+        const float nv_ = fmaf(snx, hxv, sny * hyv), nn_ = fmaf(snx, hxn, sny * hyn);
+        const float fv_ = fmaf(sfx, hxv, sfy * hyv), fn_ = fmaf(sfx, hxn, sfy * hyn);
+        float t0 = vr + V.Kv * __fdividef(fmaf(-rv, nn_ - hzn, nv_ - hzv), cn + nn_ - hzn);
+        float t1 = vr + V.Kv * __fdividef(fmaf(-rv, nn_ + hzn, nv_ + hzv), cn + nn_ + hzn);
+        float t2 = vr + V.Kv * __fdividef(fmaf(-rv, fn_ - hzn, fv_ - hzv), cn + fn_ - hzn);
+        float t3 = vr + V.Kv * __fdividef(fmaf(-rv, fn_ + hzn, fv_ + hzv), cn + fn_ + hzn);
+        sort4(t0, t1, t2, t3);
+        const Trap Tv = nc_trap(t0, t1, t2, t3);
+        const int e0 = (int)floorf(Tv.k0 + 0.5f), e1 = (int)floorf(Tv.k3 + 0.5f);
+        nc_cells<NB>(Tv, e0, e1, P.Fv);
+        P.b0 = bref + e0;
     } else {  // axial rectangle: the end points (z -+ dz/2) at the voxel's (x, y) centre
         float vlo, vhi;
         nc_pair(Kvr, rcn, rv, hzv, hzn, vr, vlo, vhi);

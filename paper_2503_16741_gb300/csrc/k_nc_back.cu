@@ -43,10 +43,10 @@ __device__ __forceinline__ float nc_taps(const NcFp<NA, NB> &P, const TIn *__res
 // Thread = voxel column (i, j) over ZT voxels; per view it forms what the
 // column shares and runs over its voxels one at a time (the per-voxel body
 // appears once in the code, which keeps the kernel within the instruction
-// cache) with the voxels' sums in shared memory.  Bound by instruction issue
-// (84 % of slots).  192^3 / 250 views FP16 SF-TR 19.8 -> 15.6 ms from forming
+// cache) with the voxels' sums in shared memory.  Bound by instruction
+// issue.  192^3 / 250 views FP16 SF-TR 19.8 -> 15.6 ms from forming
 // corner pairs with one division each and the column's share once per view;
-// 64^3 / 90 views DD 637 -> 260 us, the views split over a cluster besides.
+// 64^3 / 90 views DD 637 -> 240 us, the views split over a cluster besides.
 // RECON: the recon-mode (FBP) backprojection with the normalised footprint
 // as the interpolation: weight rc_w / depth^2 over the footprint's area x
 // height (SF-TR and DD).

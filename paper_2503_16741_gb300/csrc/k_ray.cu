@@ -170,7 +170,7 @@ __device__ __forceinline__ void slab_xy(float w, float e, float h, float &lo, fl
 // column's shadow holds at most 2 cell centres when the footprint bound is
 // below one cell (NC = 2, one group), else groups of 4.  The voxel loop is
 // not unrolled and its sums sit in shared memory.  Small volumes split the views
-// over the blocks of a cluster.  Bound by instruction issue (77 % of slots);
+// over the blocks of a cluster.  Bound by instruction issue;
 // 128^3 / 180 views: 1.97 -> 1.50 ms from the cheaper shadow (opposite corners in
 // pairs, fast reciprocals) and patches of 8 x 4 columns to a warp.
 template <bool CURVED, int ZT, int NC>

@@ -11,9 +11,10 @@
 // of its central ray through one slab -- applied once per cell after the
 // gather in the forward, and to the sinogram before the gather in the back.
 // Forward and back are gather kernels (no atomics) that evaluate the same
-// per-voxel weight functions, so they form a matched pair.  The streaming
-// forward also serves the voxel-driven projector in circular geometry (its
-// hat weights in place of the footprints; the back kernel is in k_voxel.cu).
+// per-voxel weight functions, so they form a matched pair.  SF-TR, DD and the
+// voxel-driven projector come here only for sizes that k_circ_fwd.cuh and
+// k_circ_back.cuh do not take (the voxel-driven back: k_voxel.cu); SF-TT in
+// circular flat geometry always does.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -106,9 +107,9 @@ __device__ __forceinline__ TtCol tt_col(const CtView &V, const CtGrid &g, const 
 }
 
 // rows e0 .. e0 + 3 (relative to the row of the voxel centre, whose offset
-// in it is vf) under the axial trapezoid of voxel fk, and their weights
-// (zero past the trapezoid; it spans at most 4 rows when its half height
-// bound is at most 1.5 rows)
+// in it is vf) under the axial trapezoid of voxel fk, and their weights (past
+// the trapezoid differences of equal areas, zero up to their rounding; it spans
+// at most 4 rows when its half height bound is at most 1.5 rows)
 __device__ __forceinline__ void tt_rows(const SfCol &C, const TtCol &T, float fk, float vf, int &e0,
                                         float (&Fv)[4]) {
     const float gk = fmaf(C.sv, fk, T.g0);

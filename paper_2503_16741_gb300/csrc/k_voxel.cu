@@ -1,13 +1,15 @@
 // k_voxel.cu -- voxel-driven projector (Peters 1981, cited in Sec. 2.3).
 // A voxel is a point at its centre; it is projected to the detector and
-// shared between the 2 (2D) or 4 (3D) nearest cells with bilinear weights.
+// shared between the 4 nearest cells with bilinear weights.
 // The amplitude spreads the voxel's mass over the local ray density:
-//   3D  A = dx dy dz r D^2 / (rho^3 du dv)      2D  A = dx dy r D / (rho^2 du)
+//   A = dx dy dz r D^2 / (rho^3 du dv)
 // with r = |X - s|, rho = (X - s).n (flat) or the distance of X from the
 // source axis (curved), D = source-detector distance (radius if curved).
 // The back kernel is the classic voxel-driven backprojector; the forward
-// kernels are its exact adjoint in gather form: the streaming forward of
-// k_sf.cu in circular geometry, vx_fwd_nc below in non-circular geometry.
+// kernels are its exact adjoint in gather form.  Circular geometry takes
+// k_circ_fwd.cuh and k_circ_back.cuh; here are the non-circular kernels and the
+// back for detectors of fewer than 8 cells and voxels of 8 rows and more (fan
+// beam: k_fan.cu).
 #include "ct_device.cuh"
 #include "ct_launch.h"
 
@@ -210,8 +212,8 @@ vx_back_nc(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ s
 
 // ------------------------------------------------------------ forward (gather)
 // Non-circular geometry: cell (a, b) receives the voxels whose centre
-// projects within one cell of it (circular geometries take the streaming
-// forward of k_sf.cu, which shares each column's u position down z).
+// projects within one cell of it (circular geometries share each column's u
+// position down z, k_circ_fwd.cuh).
 template <typename TIn>
 __global__ void __launch_bounds__(256)
 vx_fwd_nc(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol,
