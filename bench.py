@@ -51,14 +51,14 @@ WORKLOAD = ("3D circular cone-beam SF-TR forward+back, 256^3 x 0.5 mm FP32 volum
 SF_FLOPS_PER_UPDATE = 30.0
 FP32_LANES = 128  # FP32 FMA lanes per SM (Blackwell)
 
-# Counters of one `ncu --set full` capture of each kernel on this workload
+# Counters of one ncu capture of each kernel on this workload
 # (per launch): DRAM read + write bytes, L2 (lts__t_sectors x 32) bytes and the
 # L2 throughput peak implied by its percent-of-peak counter; src = sha256
 # prefix of the kernel's source at capture time (the bench reports null once the
 # source differs).
 NCU = {
-    "sf_fwd": {"dram_bytes": 1495.7e6, "l2_bytes": 28.577e9, "l2_peak_gbs": 36388.0, "src": "e6fc26b8654f6756"},
-    "sf_back": {"dram_bytes": 379.7e6, "l2_bytes": 11.380e9, "l2_peak_gbs": 36409.0, "src": "fd28c3c0410b5e93"},
+    "sf_fwd": {"dram_bytes": 1473.6e6, "l2_bytes": 28.594e9, "l2_peak_gbs": 36405.0, "src": "edd20dc5e8b8edc0"},
+    "sf_back": {"dram_bytes": 373.4e6, "l2_bytes": 11.355e9, "l2_peak_gbs": 36396.0, "src": "d448765ab2560a15"},
 }
 
 

@@ -19,7 +19,7 @@
 // Batch items go in pairs that share each footprint.
 // Measured against the circular kernels with nz = nv = 1 that served fan beam
 // before (forward + back of one pass): 128 x 128, 180 views, ray-driven
-// forward and voxel-driven back 310 -> 38 us; 512 x 512, 720 views, FBP
+// forward and voxel-driven back 310 -> 36 us; 512 x 512, 720 views, FBP
 // 2058 -> 380 us (436 us with one pixel to a thread); 2 images of 301 x 301,
 // 217 views, SF forward and back 4460 -> 625 us (1192 us before the pairs and
 // the cheaper footprint).

@@ -259,7 +259,7 @@ nc_fwd(CtGrid g, const CtView *__restrict__ views, const TIn *__restrict__ vol, 
 // but adds each weight once, where a gathering thread visits every voxel that
 // might reach its cells (five visits of 16 products per update for about eight
 // non-zero weights).  192^3 / 250 views / 384^2 FP16 SF-TR: gather 52.8 ms, tile
-// sums 27.2 ms (bound by L1 and instruction issue); 64^3 / 90 views DD 924 -> 415 us.
+// sums 27.4 ms (bound by instruction issue and L1); 64^3 / 90 views DD 924 -> 390 us.
 template <int NA, int NB> struct ScTile {
     static constexpr int kMc = NA - 1, kMr = NB - 1;  // margins
     static constexpr int kPitch = (32 + 2 * kMc) | 1;
